@@ -201,7 +201,7 @@ size_t carve(const yy_config* c, char* base, Bufs<T>* out) {
         b.nu_chunk = cv.take<float>((size_t)n_pad * (r_pad / kColAlign) * sizeof(float));
     // plain form of a filter with fewer than two target blocks of 64 per SM: its source
     // ranges' partial states
-    if ((c->precision == YY_PREC_FP32 || c->precision == YY_PREC_FP64) && n_pad < 2 * 152 * 64)
+    if ((c->precision == YY_PREC_FP32 || c->precision == YY_PREC_FP64) && n_pad < 2 * kSms * 64)
         b.simt_part = cv.take<T>((size_t)n_pad * kSimtMaxSplit * kMaxScales * 2 * sizeof(T));
     if (c->precision == YY_PREC_BF16) {
         b.tc_q = cv.take<float>((size_t)n_pad * sizeof(float));
@@ -474,6 +474,7 @@ yy_status yy_create(const yy_config* cfg, void* d_workspace, size_t bytes, void*
     else carve<float>(cfg, f->ws, &f->bf);
     cudaError_t e = cudaSuccess;
     if (cfg->precision == YY_PREC_BF16) e = prepare_ksum_tc();
+    if (e == cudaSuccess && !f->fp64) e = prepare_pair();
     if (e == cudaSuccess && cfg->materialise && !f->fp64) e = prepare_op_apply();
     if (e == cudaSuccess) e = cudaMemsetAsync(d_workspace, 0, need, f->stream);
     if (e != cudaSuccess) { delete f; return YY_ERR_CUDA; }
@@ -531,7 +532,7 @@ yy_status yy_predict(yy_filter* f) {
     if (f->fp64) {
         e = cudaMemsetAsync(&f->bd.stats->clamps, 0, sizeof(unsigned), f->stream);
         int l = 0;
-        if (e == cudaSuccess) e = launch_ksum_simt<double>(f->kd, f->bd, f->stream, &l);
+        if (e == cudaSuccess) e = launch_ksum_simt(f->kd, f->bd, f->stream, &l);
         f->launches += l;
     } else if (f->use_op) {
         // materialised schedule: rebuild on the device if the node set moved, then apply
@@ -542,7 +543,7 @@ yy_status yy_predict(yy_filter* f) {
     } else if (f->cfg.precision == YY_PREC_FP32 || f->route_plain) {
         e = cudaMemsetAsync(&f->bf.stats->clamps, 0, sizeof(unsigned), f->stream);
         int l = 0;
-        if (e == cudaSuccess) e = launch_ksum_simt<float>(f->kf, f->bf, f->stream, &l);
+        if (e == cudaSuccess) e = launch_pair(f->kf, f->bf, f->stream, &l);
         f->launches += l;
     } else if (f->cfg.precision == YY_PREC_FP32_SCREEN) {
         // first pass over 64 k coordinates: k = screen_prefix, else half of the 64-chunks

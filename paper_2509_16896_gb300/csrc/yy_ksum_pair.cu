@@ -1,0 +1,131 @@
+// Plain float32 prediction (and the materialised operator's build) on the pair loop of
+// yy_pair.cuh: single filters, with and without noise coefficients.
+//
+// For every target i and scale j (tau_j = dt / 2^(j-1)), in units relative to c_ref:
+//   L_j(i) - c_ref = (C_j - c_ref) - tau_j div f(x_i)
+//                    + LSE_s [ -|u_i - tau_j f_i - u_s|^2 / (2 tau_j) + ell_s ],
+//   C_j = -(r/2) log(2 pi tau_j) + log w_q,
+// which is log sum_s K_{tau_j}(x_i, x_s) w_q e^{ell_s} for the first-order kernel of
+// eq. kernel ("First-Order Kernel Construction") after completing the square:
+//   -|x-y|^2/(2 tau) - (y-x).f(x) - tau(div f + |f|^2/2) = -|x - tau f(x) - y|^2/(2 tau) - tau div f,
+//   |u_i - tau f_i - u_s|^2 = S1 - 2 tau S2 + tau^2 |f_i|^2,  S1 = |D|^2, S2 = D.f_i, D = u_i - u_s,
+// so one pass over the coordinates serves all N scales.  The N terms are combined with the
+// identity term of eq. general_kernel by a signed log-sum-exp; a non-positive total gives
+// -inf (counted).  Noise coefficients (diagonal): S1 and S2 take the target's metric a(x_i)^+,
+// |f_i|^2 likewise, and -1/2 log det_+ a(x_i) is added in the combination.
+#include <algorithm>
+
+#include "yy_pair.cuh"
+
+namespace yy {
+
+namespace {
+
+using namespace pair;
+
+template <int N, bool NOISE>
+__global__ void __launch_bounds__(THREADS, BLOCKS_PER_SM)
+    k_pair(const __grid_constant__ Consts<float> k, const __grid_constant__ Bufs<float> b, int nsplit) {
+    extern __shared__ __align__(16) float pair_smem[];
+    block<N, NOISE, false>(k, b, k.row0 + (long long)(blockIdx.x / nsplit) * BM, (int)(blockIdx.x % nsplit), nsplit,
+                           pair_smem);
+}
+
+template <int N, bool NOISE>
+__global__ void __launch_bounds__(256) k_pair_merge(const __grid_constant__ Consts<float> k,
+                                                    const __grid_constant__ Bufs<float> b, int nsplit) {
+    const long long i = k.row0 + (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= k.row1 || i >= k.n) return;
+    merge_row<N, NOISE>(k, b, i, nsplit);
+}
+
+// Materialised operator: built only when the node set moved since the last build (the flag
+// is set by restarts and state changes, cleared by the apply), unless forced.
+template <int N>
+__global__ void __launch_bounds__(THREADS, BLOCKS_PER_SM)
+    k_op_build(const __grid_constant__ Consts<float> k, const __grid_constant__ Bufs<float> b, int nsplit, int force) {
+    if (!force && b.stats->op_stale == 0) return;
+    extern __shared__ __align__(16) float pair_smem[];
+    block<N, false, true>(k, b, k.row0 + (long long)(blockIdx.x / nsplit) * BM, (int)(blockIdx.x % nsplit), nsplit,
+                          pair_smem);
+}
+
+template <int N>
+cudaError_t set_attr_n() {
+    const auto a = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    cudaError_t e = cudaFuncSetAttribute(k_pair<N, false>, a, (int)smem_bytes<N, false, false>());
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_pair<N, true>, a, (int)smem_bytes<N, true, false>());
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_op_build<N>, a, (int)smem_bytes<N, false, true>());
+    return e;
+}
+
+template <int N, bool NOISE>
+cudaError_t launch_n(const Consts<float>& k, const Bufs<float>& b, long long rows, int S, cudaStream_t s) {
+    const unsigned grid = (unsigned)((rows + BM - 1) / BM * S);
+    k_pair<N, NOISE><<<grid, THREADS, smem_bytes<N, NOISE, false>(), s>>>(k, b, S);
+    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess && S > 1) {
+        k_pair_merge<N, NOISE><<<(unsigned)((rows + 127) / 128), 128, 0, s>>>(k, b, S);
+        e = cudaGetLastError();
+    }
+    return e;
+}
+
+}  // namespace
+
+// Opts the kernels into their shared-memory sizes on the current device (at creation, so
+// that no attribute call happens during stream capture).
+cudaError_t prepare_pair() {
+    cudaError_t e = set_attr_n<1>();
+    if (e == cudaSuccess) e = set_attr_n<2>();
+    if (e == cudaSuccess) e = set_attr_n<3>();
+    if (e == cudaSuccess) e = set_attr_n<4>();
+    return e;
+}
+
+// Source ranges per target row (at most kSimtMaxSplit, none beyond the source groups): two
+// blocks of 64 targets per SM where the filter has few targets and the workspace holds the
+// partial states.
+static int pair_splits(const Consts<float>& k, const Bufs<float>& b, long long rows) {
+    if (!b.simt_part) return 1;
+    const long long blocks = (rows + 63) / 64;
+    long long sp = (2 * kSms + blocks - 1) / blocks;
+    sp = std::min<long long>(sp, kSimtMaxSplit);
+    sp = std::min<long long>(sp, k.n_pad / 64);
+    return (int)std::max<long long>(sp, 1);
+}
+
+cudaError_t launch_pair(const Consts<float>& k, const Bufs<float>& b, cudaStream_t s, int* launches) {
+    const long long rows = k.row1 - k.row0;
+    if (rows <= 0) return cudaSuccess;
+    const int S = pair_splits(k, b, rows);
+    const bool noise = k.noise == YY_NOISE_DIAG;
+    if (launches) *launches += S > 1 ? 2 : 1;
+    switch (k.N) {
+        case 1: return noise ? launch_n<1, true>(k, b, rows, S, s) : launch_n<1, false>(k, b, rows, S, s);
+        case 2: return noise ? launch_n<2, true>(k, b, rows, S, s) : launch_n<2, false>(k, b, rows, S, s);
+        case 3: return noise ? launch_n<3, true>(k, b, rows, S, s) : launch_n<3, false>(k, b, rows, S, s);
+        case 4: return noise ? launch_n<4, true>(k, b, rows, S, s) : launch_n<4, false>(k, b, rows, S, s);
+    }
+    return cudaErrorInvalidValue;
+}
+
+cudaError_t launch_op_build(const Consts<float>& k, const Bufs<float>& b, bool force, cudaStream_t s) {
+    if (!b.op) return cudaErrorInvalidValue;
+    const long long rows = k.row1 - k.row0;
+    if (rows <= 0) return cudaSuccess;
+    // entries are independent, so the source ranges only balance the SMs
+    const int S = (int)std::max<long long>(1, std::min<long long>(8, k.n_pad / 512));
+    const unsigned grid = (unsigned)((rows + BM - 1) / BM * S);
+    const int f = force ? 1 : 0;
+    switch (k.N) {
+        case 1: k_op_build<1><<<grid, THREADS, smem_bytes<1, false, true>(), s>>>(k, b, S, f); break;
+        case 2: k_op_build<2><<<grid, THREADS, smem_bytes<2, false, true>(), s>>>(k, b, S, f); break;
+        case 3: k_op_build<3><<<grid, THREADS, smem_bytes<3, false, true>(), s>>>(k, b, S, f); break;
+        case 4: k_op_build<4><<<grid, THREADS, smem_bytes<4, false, true>(), s>>>(k, b, S, f); break;
+        default: return cudaErrorInvalidValue;
+    }
+    return cudaGetLastError();
+}
+
+}  // namespace yy

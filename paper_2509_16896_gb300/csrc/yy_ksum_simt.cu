@@ -1,4 +1,6 @@
-// Prediction step, plain form on the FMA pipes (float32 or float64).
+// Prediction step on the FMA pipes: the plain form in float64 (and in float32 for batches),
+// the screened float32 form and the materialised operator's apply.  The plain float32 form of a
+// single filter is in yy_ksum_pair.cu.
 //
 // For every target i and scale j (tau_j = dt / 2^(j-1)), in units relative to c_ref:
 //   L_j(i) - c_ref = (C_j - c_ref) - tau_j div f(x_i)
@@ -52,13 +54,10 @@ template <> __device__ __forceinline__ double exp_fast<double>(double x) { retur
 // NOISE (diagonal noise coefficients): the squared distance and the drift's inner product
 // take the target's metric a(x_i)^+, S1 = sum_d m_d D_d^2, S2 = sum_d m_d D_d f_d, with
 // |f_i|^2 in the same metric (nf) and -1/2 log det_+ a(x_i) added in the combination.
-// OPBUILD (float32): the materialised operator -- every pair's score without the source
-// weight, A_j(i, s) = -S1 / (2 tau_j) + S2 - tau_j |f_i|^2 / 2, is written to b.op instead of
-// being accumulated.
 // split / nsplit (plain form of a filter with few target blocks): this block sweeps only the
 // split-th of nsplit equal ranges of source tiles and stores its rows' partial (max, sum)
 // per scale in b.simt_part; k_simt_merge combines the ranges.
-template <typename T, int N, bool SCREEN = false, bool NOISE = false, bool OPBUILD = false>
+template <typename T, int N, bool SCREEN = false, bool NOISE = false>
 __device__ __forceinline__ void ksum_simt_body(const Consts<T>& k, const Bufs<T>& b, int rk, int bid, int k1 = 0,
                                                int split = 0, int nsplit = 1) {
     __shared__ T At[BK][BM];   // u of targets
@@ -210,24 +209,6 @@ __device__ __forceinline__ void ksum_simt_body(const Consts<T>& k, const Bufs<T>
                     }
             }
         }
-        if constexpr (OPBUILD) {
-            const size_t plane = (size_t)k.n_pad * (size_t)k.n_pad;
-#pragma unroll
-            for (int a = 0; a < TM; ++a) {
-                const long long i = i0 + ty * TM + a;
-#pragma unroll
-                for (int j = 0; j < N; ++j) {
-                    float4 v;
-                    v.x = (float)(fma(-S1[a][0], k.inv2tau[j], S2[a][0]) + rowc[a][j]);
-                    v.y = (float)(fma(-S1[a][1], k.inv2tau[j], S2[a][1]) + rowc[a][j]);
-                    v.z = (float)(fma(-S1[a][2], k.inv2tau[j], S2[a][2]) + rowc[a][j]);
-                    v.w = (float)(fma(-S1[a][3], k.inv2tau[j], S2[a][3]) + rowc[a][j]);
-                    *reinterpret_cast<float4*>(b.op + j * plane + (size_t)i * k.n_pad + s0 + tx * TN) = v;
-                }
-            }
-            __syncthreads();
-            continue;
-        }
         // scores and online log-sum-exp for this source tile
         T ls[TN];
 #pragma unroll
@@ -254,7 +235,6 @@ __device__ __forceinline__ void ksum_simt_body(const Consts<T>& k, const Bufs<T>
         __syncthreads();
     }
 
-    if constexpr (OPBUILD) return;
     // merge the 16 threads that share a target group (lanes differing in the low 4 bits)
 #pragma unroll
     for (int a = 0; a < TM; ++a)
@@ -335,14 +315,6 @@ __global__ void __launch_bounds__(256) k_simt_merge(Consts<T> k, Bufs<T> b, int 
 template <int N>
 __global__ void __launch_bounds__(256) k_ksum_scr32(Consts<float> k, Bufs<float> b, int rk, int k1) {
     ksum_simt_body<float, N, true>(k, b, rk, (int)(k.row0 / BM) + blockIdx.x, k1);
-}
-
-// Materialised operator: built only when the node set moved since the last build (the flag
-// is set by restarts and state changes, cleared by the apply), unless forced.
-template <int N>
-__global__ void __launch_bounds__(256) k_op_build(Consts<float> k, Bufs<float> b, int rk, int force) {
-    if (!force && b.stats->op_stale == 0) return;
-    ksum_simt_body<float, N, false, false, true>(k, b, rk, (int)(k.row0 / BM) + blockIdx.x);
 }
 
 // The apply works in base 2: with v = A + ell, e^(v - m) = 2^(v log2 e - m log2 e).
@@ -552,21 +524,6 @@ __global__ void __launch_bounds__(288) k_op_apply(Consts<float> k, Bufs<float> b
     }
 }
 
-cudaError_t launch_op_build(const Consts<float>& k, const Bufs<float>& b, bool force, cudaStream_t s) {
-    if (!b.op) return cudaErrorInvalidValue;
-    const int rk = ((k.r + BK - 1) / BK) * BK;
-    const unsigned grid = (unsigned)((k.row1 - k.row0 + BM - 1) / BM);
-    if (grid == 0) return cudaSuccess;
-    switch (k.N) {
-        case 1: k_op_build<1><<<grid, 256, 0, s>>>(k, b, rk, force ? 1 : 0); break;
-        case 2: k_op_build<2><<<grid, 256, 0, s>>>(k, b, rk, force ? 1 : 0); break;
-        case 3: k_op_build<3><<<grid, 256, 0, s>>>(k, b, rk, force ? 1 : 0); break;
-        case 4: k_op_build<4><<<grid, 256, 0, s>>>(k, b, rk, force ? 1 : 0); break;
-        default: return cudaErrorInvalidValue;
-    }
-    return cudaGetLastError();
-}
-
 namespace {
 int g_op_resident[5] = {0, 0, 0, 0, 0};   // blocks of k_op_apply<N> resident on the device at once
 }
@@ -667,7 +624,6 @@ cudaError_t launch_ksum_simt_batch(const Traj<T>* d_traj, int B, int N, long lon
     return cudaGetLastError();
 }
 template cudaError_t launch_ksum_simt_batch<float>(const Traj<float>*, int, int, long long, int, cudaStream_t, int*);
-template cudaError_t launch_ksum_simt_batch<double>(const Traj<double>*, int, int, long long, int, cudaStream_t, int*);
 
 // Source ranges per target block of the plain form: enough blocks for two per SM (at most
 // kSimtMaxSplit ranges, none beyond the source tiles), when the filter has few target
@@ -680,8 +636,7 @@ int simt_splits(long long n_pad, long long tiles, bool has_part) {
     return (int)std::max<long long>(sp, 1);
 }
 
-template <typename T>
-cudaError_t launch_ksum_simt(const Consts<T>& k, const Bufs<T>& b, cudaStream_t s, int* launches) {
+cudaError_t launch_ksum_simt(const Consts<double>& k, const Bufs<double>& b, cudaStream_t s, int* launches) {
     const int rk = ((k.r + BK - 1) / BK) * BK;
     const long long tiles = (k.row1 - k.row0 + BM - 1) / BM;   // the handle's target blocks
     if (tiles == 0) return cudaSuccess;
@@ -690,12 +645,12 @@ cudaError_t launch_ksum_simt(const Consts<T>& k, const Bufs<T>& b, cudaStream_t 
     const bool noise = (k.noise == YY_NOISE_DIAG);
 #define YY_SIMT(NN)                                                                                     \
     case NN:                                                                                            \
-        if (noise) k_ksum_simt<T, NN, true><<<grid, 256, 0, s>>>(k, b, rk, nsplit);                     \
-        else k_ksum_simt<T, NN><<<grid, 256, 0, s>>>(k, b, rk, nsplit);                                \
+        if (noise) k_ksum_simt<double, NN, true><<<grid, 256, 0, s>>>(k, b, rk, nsplit);                \
+        else k_ksum_simt<double, NN><<<grid, 256, 0, s>>>(k, b, rk, nsplit);                           \
         if (nsplit > 1) {                                                                               \
             const unsigned mg = (unsigned)((k.row1 - k.row0 + 255) / 256);                              \
-            if (noise) k_simt_merge<T, NN, true><<<mg, 256, 0, s>>>(k, b, nsplit);                      \
-            else k_simt_merge<T, NN><<<mg, 256, 0, s>>>(k, b, nsplit);                                 \
+            if (noise) k_simt_merge<double, NN, true><<<mg, 256, 0, s>>>(k, b, nsplit);                 \
+            else k_simt_merge<double, NN><<<mg, 256, 0, s>>>(k, b, nsplit);                            \
         }                                                                                               \
         break;
     switch (k.N) {
@@ -709,7 +664,5 @@ cudaError_t launch_ksum_simt(const Consts<T>& k, const Bufs<T>& b, cudaStream_t 
     if (launches) *launches += (nsplit > 1) ? 2 : 1;
     return cudaGetLastError();
 }
-template cudaError_t launch_ksum_simt<float>(const Consts<float>&, const Bufs<float>&, cudaStream_t, int*);
-template cudaError_t launch_ksum_simt<double>(const Consts<double>&, const Bufs<double>&, cudaStream_t, int*);
 
 }  // namespace yy

@@ -1,0 +1,51 @@
+"""The float32 pair loop (packed, 32 x 128 tiles, 16-coordinate stages) at the edges of its
+tiles: target counts around 32, source counts around the groups of 64 and tiles of 128 and
+the source ranges, coordinate counts around a stage, every number of scales, with and
+without noise coefficients -- each predicted log-weight against the FP64 oracle within the
+float32 bar of the step tests, 1e-5 relative, plus what the multi-scale combination
+amplifies (`combination_err_ok`)."""
+import numpy as np
+import pytest
+
+from ._helpers import combination_err_ok, oracle_problem, sobol_inputs
+
+pytestmark = pytest.mark.gpu
+
+NOISE = dict(u=0.7, u_kappa=0.8, u_zero=0, v=1.3, v_kappa=0.5)
+
+
+@pytest.mark.parametrize("r,n,N,noise", [(1, 2, 1, False), (2, 31, 2, False), (15, 33, 3, False), (16, 64, 4, False),
+                                         (17, 65, 1, False), (31, 127, 2, False), (32, 129, 3, False),
+                                         (33, 257, 2, False), (63, 320, 2, False), (64, 321, 1, False),
+                                         (65, 1025, 2, False), (129, 577, 3, False), (8, 20000, 2, False),
+                                         (5, 63, 2, True), (16, 129, 1, True), (49, 700, 4, True)])
+def test_prediction_at_tile_edges(yy_lib, r, n, N, noise):
+    from oracle import filter as F
+    from paper_2509_16896_gb300 import binding
+    nz = NOISE if noise else None
+    R = 0.3 if r > 8 else 1.0
+    f = binding.Filter(binding.make_config(model="cubic", r=r, n=n, dt=0.01, R=R, n_scales=N, precision="f32", noise=nz))
+    poly, scr = sobol_inputs(r, 40 + r)
+    f.init_nodes(poly, scr, np.zeros(r))
+    u, _ = f.get_nodes()
+    p = oracle_problem("cubic", r, n, 0.01, R, N, noise=nz)
+    rng = np.random.default_rng(r * 1000 + n)
+    centre = rng.standard_normal(r)
+    # weights of a posterior: a few nats apart, some nodes without weight
+    lw = (-2.0 * rng.random(n) - np.log(n)).astype(np.float32)
+    lw[rng.random(n) < 0.05] = -np.inf
+    lw[0] = 0.0
+    f.set_state(centre, lw, 0.0, 1)
+    f.predict()
+    pred, off = f.get_log_weights()
+    prep = F.prepare(p, u, centre)
+    lw64 = lw.astype(np.float64)
+    Lj = F.kernel_lse(p, prep, lw64)
+    ref, _ = F.combine(p, Lj, lw64, prep.mask)
+    got = pred.astype(np.float64) + off
+    # a row whose combination is within float32 error of zero may clamp on one side only
+    both = np.isfinite(got) == np.isfinite(ref)
+    assert both.mean() >= 0.99, np.nonzero(~both)[0][:5]
+    ok, kappa = combination_err_ok(got[both], ref[both], Lj[both], p.coef, lw64[both], 1e-5)
+    print(f"r={r} n={n} N={N} noise={noise}: largest condition number {kappa:.1f}")
+    assert ok
