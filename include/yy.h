@@ -83,7 +83,8 @@ typedef enum { YY_MODEL_CUBIC = 0, YY_MODEL_LINEAR = 1, YY_MODEL_PAPER_E1 = 2 } 
 typedef enum { YY_NODES_SOBOL = 0, YY_NODES_HALTON = 1, YY_NODES_FAURE = 2 } yy_nodes;
 
 /* Arithmetic of the prediction step.  FP64: every step in float64.  FP32: exact
- * float32 differences over every pair.  BF16: a tcgen05 BF16 Gram product screens out pairs
+ * float32 differences over every pair (at r >= 128 a pair whose term is provably zero in
+ * float32 next to the largest of its row is not summed to the end).  BF16: a tcgen05 BF16 Gram product screens out pairs
  * whose kernel term is provably negligible, and the remaining pairs are evaluated exactly
  * in float32 (results agree with FP32 within float32 rounding).  FP32_SCREEN: the same kind
  * of screen on the FMA pipes, no tensor cores: a tile of 64 x 64 pairs is skipped when the

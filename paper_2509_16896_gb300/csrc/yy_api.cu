@@ -203,6 +203,8 @@ size_t carve(const yy_config* c, char* base, Bufs<T>* out) {
     // ranges' partial states
     if ((c->precision == YY_PREC_FP32 || c->precision == YY_PREC_FP64) && n_pad < 2 * kSms * 64)
         b.simt_part = cv.take<T>((size_t)n_pad * kSimtMaxSplit * kMaxScales * 2 * sizeof(T));
+    if (c->precision == YY_PREC_FP32 || c->precision == YY_PREC_BF16)
+        b.pair_ref = cv.take<float>((size_t)n_pad * kMaxScales * sizeof(float));
     if (c->precision == YY_PREC_BF16) {
         b.tc_q = cv.take<float>((size_t)n_pad * sizeof(float));
         b.tc_q1 = cv.take<float>((size_t)n_pad * sizeof(float));

@@ -146,6 +146,8 @@ struct Bufs {
     float* tc_part;       // [n_pad][8][4][2] partial (max, sum) of split work items
     T* simt_part;         // [n_pad][kSimtMaxSplit][kMaxScales][2] plain forms: partial (max, sum)
                           // of each source range (filters with few target blocks only)
+    float* pair_ref;      // [n_pad][kMaxScales] plain float32 form of long rows: lower bounds of the
+                          // rows' largest scores
     int4* tc_items;       // single-filter work list (target tile, split, nsplit)
     int* tc_cta_start;    // [tc_grid + 1]
     int tc_grid;          // persistent CTAs of the single-filter prediction

@@ -31,6 +31,69 @@ __global__ void __launch_bounds__(THREADS, BLOCKS_PER_SM)
                            pair_smem);
 }
 
+// The same with terms that cannot count left out (see block); flags: per target block of 32, a
+// bit per tile of 128 sources (fwords words per block), or nullptr.
+template <int N>
+__global__ void __launch_bounds__(THREADS, BLOCKS_PER_SM)
+    k_pair_skip(const __grid_constant__ Consts<float> k, const __grid_constant__ Bufs<float> b, int nsplit, float gap,
+                const uint32_t* __restrict__ flags, int fwords) {
+    extern __shared__ __align__(16) float pair_smem[];
+    const long long i0 = k.row0 + (long long)(blockIdx.x / nsplit) * BM;
+    block<N, false, false, true>(k, b, i0, (int)(blockIdx.x % nsplit), nsplit, pair_smem, gap,
+                                 flags ? flags + (size_t)(i0 / BM) * fwords : nullptr);
+}
+
+// Lower bounds of every target row's largest score, per scale: the larger of the row's own
+// term (u_i - u_i = 0) and its exact score against the live source of the largest log-weight.
+// Each block finds that source for itself (n words from L2); then one warp per row.
+template <int N>
+__global__ void __launch_bounds__(256) k_pair_ref(const __grid_constant__ Consts<float> k,
+                                                  const __grid_constant__ Bufs<float> b) {
+    __shared__ float sm[8];
+    __shared__ long long si[8];
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    float m = -INFINITY;
+    long long top = -1;
+    for (long long s = threadIdx.x; s < k.n; s += blockDim.x) {
+        const float v = b.mask[s] ? -INFINITY : b.logw[s];
+        if (v > m) { m = v; top = s; }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const float m2 = __shfl_xor_sync(0xffffffffu, m, o);
+        const long long t2 = __shfl_xor_sync(0xffffffffu, top, o);
+        if (m2 > m || (m2 == m && t2 > top)) { m = m2; top = t2; }
+    }
+    if (lane == 0) { sm[wib] = m; si[wib] = top; }
+    __syncthreads();
+    for (int w = 0; w < 8; ++w)
+        if (sm[w] > m || (sm[w] == m && si[w] > top)) { m = sm[w]; top = si[w]; }
+    const float* us = b.u + (size_t)max(top, 0ll) * k.r_pad;
+    for (long long i = k.row0 + (long long)blockIdx.x * 8 + wib; i < k.row1; i += (long long)gridDim.x * 8) {
+        const float* ui = b.u + (size_t)i * k.r_pad;
+        const float* fi = b.f + (size_t)i * k.r_pad;
+        float s1 = 0.f, s2 = 0.f;
+        for (int d = lane; d < k.r; d += 32) {
+            const float dl = ui[d] - us[d];
+            s1 = fmaf(dl, dl, s1);
+            s2 = fmaf(dl, fi[d], s2);
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+            s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+        }
+        if (lane == 0) {
+            const float nf = b.nf[i], li = b.logw[i];
+#pragma unroll
+            for (int j = 0; j < N; ++j) {
+                const float rc = -0.5f * k.tau[j] * nf;
+                b.pair_ref[(size_t)i * kMaxScales + j] = fmaxf(rc + li, fmaf(-s1, k.inv2tau[j], s2) + (rc + m));
+            }
+        }
+    }
+}
+
 template <int N, bool NOISE>
 __global__ void __launch_bounds__(256) k_pair_merge(const __grid_constant__ Consts<float> k,
                                                     const __grid_constant__ Bufs<float> b, int nsplit) {
@@ -50,19 +113,37 @@ __global__ void __launch_bounds__(THREADS, BLOCKS_PER_SM)
                           pair_smem);
 }
 
+// The skipping form: from this many coordinates (its reference pass and masks cost about 10 us,
+// and a tile is not given up before 64 coordinates: at r = 100 nothing is), up to this much
+// mask.  Measured, large-scale model at r = 1000, n = 2000, N = 2, full form 620 us per prediction:
+// weights of a restart 175 us (tiles given up after 192 to 256 coordinates; 300 us while the
+// rows' own pairs kept their tiles), weights of an update 95 us (one heavy node; 350 us before
+// thin tiles).
+constexpr int kSkipMinDim = 128;
+constexpr size_t kMaxMaskBytes = 32768;   // ranges of up to a million sources
+constexpr float kSkipGap = 110.0f;
+
 template <int N>
 cudaError_t set_attr_n() {
     const auto a = cudaFuncAttributeMaxDynamicSharedMemorySize;
     cudaError_t e = cudaFuncSetAttribute(k_pair<N, false>, a, (int)smem_bytes<N, false, false>());
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_pair<N, true>, a, (int)smem_bytes<N, true, false>());
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_pair_skip<N>, a, (int)(smem_bytes<N, false, false, true>() + kMaxMaskBytes));
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_op_build<N>, a, (int)smem_bytes<N, false, true>());
     return e;
 }
 
 template <int N, bool NOISE>
-cudaError_t launch_n(const Consts<float>& k, const Bufs<float>& b, long long rows, int S, cudaStream_t s) {
+cudaError_t launch_n(const Consts<float>& k, const Bufs<float>& b, long long rows, int S, cudaStream_t s, int* l) {
     const unsigned grid = (unsigned)((rows + BM - 1) / BM * S);
-    k_pair<N, NOISE><<<grid, THREADS, smem_bytes<N, NOISE, false>(), s>>>(k, b, S);
+    const size_t mask = 16 * sizeof(uint32_t) * (size_t)mask_words(k.n, S);
+    if (!NOISE && b.pair_ref && k.r >= kSkipMinDim && mask <= kMaxMaskBytes) {
+        k_pair_ref<N><<<(unsigned)std::min<long long>((rows + 7) / 8, 2 * kSms), 256, 0, s>>>(k, b);
+        k_pair_skip<N><<<grid, THREADS, smem_bytes<N, false, false, true>() + mask, s>>>(k, b, S, kSkipGap, nullptr, 0);
+        if (l) *l += 1;
+    } else {
+        k_pair<N, NOISE><<<grid, THREADS, smem_bytes<N, NOISE, false>(), s>>>(k, b, S);
+    }
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess && S > 1) {
         k_pair_merge<N, NOISE><<<(unsigned)((rows + 127) / 128), 128, 0, s>>>(k, b, S);
@@ -102,10 +183,10 @@ cudaError_t launch_pair(const Consts<float>& k, const Bufs<float>& b, cudaStream
     const bool noise = k.noise == YY_NOISE_DIAG;
     if (launches) *launches += S > 1 ? 2 : 1;
     switch (k.N) {
-        case 1: return noise ? launch_n<1, true>(k, b, rows, S, s) : launch_n<1, false>(k, b, rows, S, s);
-        case 2: return noise ? launch_n<2, true>(k, b, rows, S, s) : launch_n<2, false>(k, b, rows, S, s);
-        case 3: return noise ? launch_n<3, true>(k, b, rows, S, s) : launch_n<3, false>(k, b, rows, S, s);
-        case 4: return noise ? launch_n<4, true>(k, b, rows, S, s) : launch_n<4, false>(k, b, rows, S, s);
+        case 1: return noise ? launch_n<1, true>(k, b, rows, S, s, launches) : launch_n<1, false>(k, b, rows, S, s, launches);
+        case 2: return noise ? launch_n<2, true>(k, b, rows, S, s, launches) : launch_n<2, false>(k, b, rows, S, s, launches);
+        case 3: return noise ? launch_n<3, true>(k, b, rows, S, s, launches) : launch_n<3, false>(k, b, rows, S, s, launches);
+        case 4: return noise ? launch_n<4, true>(k, b, rows, S, s, launches) : launch_n<4, false>(k, b, rows, S, s, launches);
     }
     return cudaErrorInvalidValue;
 }

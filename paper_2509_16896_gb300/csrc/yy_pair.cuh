@@ -47,11 +47,18 @@ template <bool NOISE>
 __host__ __device__ constexpr int stage_words() {
     return BK * ((NOISE ? 3 : 2) * AS + BS);
 }
+// Skipping form: words of a chain's mask, one bit per group of 64 sources of a range.
+__host__ __device__ __forceinline__ int mask_words(long long n, int nsplit) {
+    const long long groups = (n + 63) / 64;
+    return (int)(((groups + nsplit - 1) / nsplit + 31) / 32);
+}
 // Two stages | log-sum-exp states per thread [TM][N][2][THREADS] | source terms of two tiles |
-// |f|^2 of the targets.
-template <int N, bool NOISE, bool OP>
+// |f|^2 of the targets | skipping form: thresholds [BM][N], group tables of two tiles [2][2][16],
+// four words, chain masks [16][mask_words].
+template <int N, bool NOISE, bool OP, bool SKIP = false>
 __host__ __device__ constexpr size_t smem_bytes() {
-    return sizeof(float) * (2 * (size_t)stage_words<NOISE>() + (OP ? 0 : TM * N * 2 * THREADS) + 2 * BN + BM);
+    return sizeof(float) * (2 * (size_t)stage_words<NOISE>() + (OP ? 0 : TM * N * 2 * THREADS) + 2 * BN + BM +
+                            (SKIP ? BM * N + 2 * 2 * 16 + 4 : 0));
 }
 
 __device__ __forceinline__ void cp4(float* dst, const float* src) {
@@ -103,13 +110,65 @@ __device__ __forceinline__ float max_nan(float a, float b) {
 // denormal's half).
 constexpr float kZeroGap = 105.0f;
 
+constexpr int kThinGroups = 2;
+// S1 and S2 of one pair over all coordinates in increasing order, loads a stage ahead.
+__device__ __forceinline__ void pair_sums_thread(const float* __restrict__ ut, const float* __restrict__ ft,
+                                                 const float* __restrict__ us, int r_pad, float& s1, float& s2) {
+    constexpr int Q = 4;   // float4 per stage and operand
+    float4 a[Q], f[Q], c[Q];
+    auto get = [&](int d) {
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            a[q] = *reinterpret_cast<const float4*>(ut + d + 4 * q);
+            f[q] = *reinterpret_cast<const float4*>(ft + d + 4 * q);
+            c[q] = *reinterpret_cast<const float4*>(us + d + 4 * q);
+        }
+    };
+    s1 = s2 = 0.f;
+    get(0);
+    for (int d = 0; d < r_pad; d += 4 * Q) {   // padded coordinates are zero in all three
+        float4 x[Q], y[Q], z[Q];
+#pragma unroll
+        for (int q = 0; q < Q; ++q) { x[q] = a[q]; y[q] = f[q]; z[q] = c[q]; }
+        if (d + 4 * Q < r_pad) get(d + 4 * Q);
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            const float xs[4] = {x[q].x, x[q].y, x[q].z, x[q].w}, ys[4] = {y[q].x, y[q].y, y[q].z, y[q].w};
+            const float zs[4] = {z[q].x, z[q].y, z[q].z, z[q].w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const float dl = xs[e] - zs[e];
+                s1 = fmaf(dl, dl, s1);
+                s2 = fmaf(dl, ys[e], s2);
+            }
+        }
+    }
+}
+
 // One block: targets i0 .. i0 + BM - 1 against the groups of 64 sources in the range [split /
 // nsplit, (split + 1) / nsplit), TN / 4 groups per source tile.  nsplit > 1: the rows' (max,
 // sum) go to b.simt_part and a merge kernel applies the combination.  OP: every pair's score
-// without the source weight, A_j(i, s) = -S1 / (2 tau_j) + S2 - tau_j |f_i|^2 / 2, is written to b.op instead.
-template <int N, bool NOISE, bool OP>
+// without the source weight, A_j(i, s) = -S1 / (2 tau_j) + S2 - tau_j |f_i|^2 / 2, is written to
+// b.op instead.
+//
+// SKIP: terms that provably cannot count are not evaluated.  b.pair_ref[i][j] is a lower bound
+// of row i's largest score at scale j (k_pair_ref); a pair whose score is below it by more than
+// gap at every scale is dropped.  Since a score is ell_s minus a sum of squares over the
+// coordinates, two bounds need no slack but rounding's (gap has 5 nats to spare):
+//   - a chain's group of 4 sources is left out when its largest ell_s is below the block's lowest
+//     threshold (weights spread over many nats: the large-scale model after an update); the
+//     remaining groups of a chain keep their order;
+//   - a tile is given up when, every 64 coordinates, -S1 / (2 tau_j) + S2 + ell_s of every pair is
+//     below its row's threshold (a row's own pair, D = 0, aside: its score is known).
+// A tile of one or two groups (one heavy node) is taken by one thread per target and source:
+// with the full tile's loop its few blocks would wait out one stage after the other.
+// With gap = 110 every dropped term is zero in float32 next to the row's largest: the row's sum
+// is bit for bit that of the full evaluation.  flags != nullptr: only groups of tiles
+// flagged for this target block ([tile of 128 sources] bits) are taken.
+template <int N, bool NOISE, bool OP, bool SKIP = false>
 __device__ __forceinline__ void block(const Consts<float>& k, const Bufs<float>& b, long long i0, int split,
-                                      int nsplit, float* smem) {
+                                      int nsplit, float* smem, float gap = 0.f, const uint32_t* flags = nullptr) {
+    static_assert(!SKIP || (!NOISE && !OP), "the skipping form is the plain one");
     constexpr int SW = stage_words<NOISE>();
     constexpr int RP = TM / 2;   // row pairs per thread
     float* st0 = smem;
@@ -122,7 +181,15 @@ __device__ __forceinline__ void block(const Consts<float>& k, const Bufs<float>&
     const long long groups = (k.n + 63) / 64;
     const long long s_begin = (groups * split / nsplit) * 64;
     const long long s_end = min(k.n, (groups * (split + 1) / nsplit) * 64);
-    const int nt = s_end > s_begin ? (int)((s_end - s_begin + BN - 1) / BN) : 0;   // source tiles
+    int nt = s_end > s_begin ? (int)((s_end - s_begin + BN - 1) / BN) : 0;   // source tiles
+    float* thr = nfs + BM;                                               // [BM][N]
+    int* grp = reinterpret_cast<int*>(thr + (SKIP ? BM * N : 0));        // [2][2][16]
+    int* gcnt = grp + 64;                                                // [2]: groups of two tiles
+    float* red = reinterpret_cast<float*>(gcnt + 2);                     // [2]
+    uint32_t* cmask = reinterpret_cast<uint32_t*>(red + 2);              // [16][mw]
+    const int mw = SKIP ? mask_words(k.n, nsplit) : 0;
+    uint32_t mword = 0u;   // thread tid < 16: the rest of chain tid's current mask word
+    int mpos = -1;
 
     for (int r = tid; r < BM; r += THREADS) nfs[r] = (i0 + r < k.n) ? b.nf[i0 + r] : 0.f;
     if constexpr (!OP) {
@@ -151,6 +218,18 @@ __device__ __forceinline__ void block(const Consts<float>& k, const Bufs<float>&
             if constexpr (NOISE) { cp4(M + lc * AS + lr + 8 * q, pm); pm += step; }
         }
         // rows past the range belong to others and carry no weight; none past n_pad is read
+        if constexpr (SKIP) {
+            const int* gt = grp + (t & 1) * 32;
+            const float* ps = b.u + (size_t)s_begin * rp + c * BK + lc;
+#pragma unroll
+            for (int q = 0; q < BN / 8; ++q) {
+                const int j = lr + 8 * q;
+                const int g = max(gt[(j >> 6) * 16 + ((j & 63) >> 2)], 0);
+                cp4(B + lc * BS + j, ps + (size_t)(g * 64 + (j & 63)) * rp);
+            }
+            cp_commit();
+            return;
+        }
         const long long s0 = s_begin + (long long)t * BN;
         const float* ps = b.u + (size_t)(s0 + lr) * rp + c * BK + lc;
         const int rows = (int)min((long long)BN, k.n_pad - s0);   // BN or 64 (uniform)
@@ -160,28 +239,159 @@ __device__ __forceinline__ void block(const Consts<float>& k, const Bufs<float>&
         cp_commit();
     };
     auto source_term = [&](int t) -> float {   // of this thread's source (tid < BN) of tile t
-        const long long s = s_begin + (long long)t * BN + tid;
+        long long s = s_begin + (long long)t * BN + tid;
+        if constexpr (SKIP) {
+            const int g = grp[(t & 1) * 32 + (tid >> 6) * 16 + ((tid & 63) >> 2)];
+            s = g < 0 ? s_end : s_begin + (long long)g * 64 + (tid & 63);
+        }
         return (tid < BN && s < s_end && !b.mask[s]) ? b.logw[s] : -INFINITY;
     };
+    // SKIP: the next two groups of every chain, for tile t (threads 0..15)
+    auto next_groups = [&](int t) {
+        if (tid >= 16) return;
+        int cnt = 0;
+#pragma unroll
+        for (int g = 0; g < 2; ++g) {
+            while (mword == 0u && mpos + 1 < mw) mword = cmask[tid * mw + ++mpos];
+            int v = -1;
+            if (mword != 0u) {
+                v = mpos * 32 + __ffs(mword) - 1;
+                mword &= mword - 1u;
+            }
+            grp[(t & 1) * 32 + g * 16 + tid] = v;
+            cnt += __popc(__ballot_sync(0xffffu, v >= 0));
+        }
+        if (tid == 0) gcnt[t & 1] = cnt;
+    };
+    // a tile of so few groups that one thread per target and source takes it
+    auto thin = [&](int t) -> bool { return SKIP && gcnt[t & 1] <= kThinGroups; };
+    if constexpr (SKIP) {
+        // thresholds of the rows and the lowest of them
+        float lo = INFINITY;
+        if (tid < BM) {
+            const long long i = i0 + tid;
+            const bool target = i < k.n && !b.mask[i];
+#pragma unroll
+            for (int j = 0; j < N; ++j) {
+                const float v = target ? b.pair_ref[(size_t)i * kMaxScales + j] - gap : INFINITY;
+                thr[tid * N + j] = v;
+                lo = (v != v) ? -INFINITY : fminf(lo, v);   // an undefined bound drops nothing
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+            if (tid == 0) red[0] = lo;
+        }
+        for (int w = tid; w < 16 * mw; w += THREADS) cmask[w] = 0u;
+        __syncthreads();
+        lo = red[0];
+        // the chains' groups that can count, one group of 64 sources per warp at a time
+        const int lane = tid & 31, ng = (int)((s_end - s_begin + 63) / 64);
+        for (int g = tid >> 5; g < ng; g += THREADS / 32) {
+            const long long s0 = s_begin + (long long)g * 64;
+            if (flags && !((flags[(s0 >> 7) >> 5] >> ((s0 >> 7) & 31)) & 1u)) continue;
+            bool act = false;
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const long long s = s0 + 2 * lane + e;
+                const float v = (s < s_end && !b.mask[s]) ? b.logw[s] : -INFINITY;
+                act |= v != -INFINITY && !(v < lo);
+            }
+            const uint32_t bal = __ballot_sync(0xffffffffu, act);
+            if (lane < 16 && ((bal >> (2 * lane)) & 3u)) atomicOr(&cmask[lane * mw + (g >> 5)], 1u << (g & 31));
+        }
+        __syncthreads();
+        if (tid < 32) {   // tiles: two groups of each chain per tile
+            int c = 0;
+            if (tid < 16)
+                for (int w = 0; w < mw; ++w) c += __popc(cmask[tid * mw + w]);
+            c = __reduce_max_sync(0xffffffffu, c);
+            if (tid == 0) red[1] = __int_as_float((c + 1) / 2);
+        }
+        next_groups(0);
+        __syncthreads();
+        nt = __float_as_int(red[1]);
+    }
 
+    // which of the thread's two groups of tile t holds its own target rows (-1: neither; rows and
+    // groups are aligned to 4)
+    auto own_group = [&](int t) -> int {
+        const long long row = i0 + ty * 4 - s_begin;
+#pragma unroll
+        for (int g = 0; g < 2; ++g) {
+            const int v = grp[(t & 1) * 32 + g * 16 + tx];
+            if (v >= 0 && (long long)v * 64 + tx * 4 == row) return g;
+        }
+        return -1;
+    };
+    // four scores into state sp of a chain (maximum, sum)
+    auto add4 = [&](float* sp, const float (&sc)[4]) {
+        float tmax = max_nan(max_nan(sc[0], sc[1]), max_nan(sc[2], sc[3]));
+        float mx = sp[0];
+        // every term zero in float32 (a NaN compares false and is taken in)
+        if (tmax < mx - kZeroGap) return;
+        if (tmax != tmax) tmax = fmaxf(fmaxf(sc[0], sc[1]), fmaxf(sc[2], sc[3]));
+        if (!(tmax > -INFINITY)) return;   // no live source
+        float sm = sp[THREADS];
+        if (tmax > mx) {
+            sm = (mx == -INFINITY) ? 0.f : sm * exp_hw(mx - tmax);
+            mx = tmax;
+        }
+#pragma unroll
+        for (int c = 0; c < 4; ++c) sm += exp_hw(sc[c] - mx);
+        sp[0] = mx;
+        sp[THREADS] = sm;
+    };
     if (nt > 0) {
-        load(0, 0, 0);
+        if (!thin(0)) load(0, 0, 0);
         if (tid < BN) lsrc[tid] = source_term(0);
     }
     int buf = 0;
     for (int t = 0; t < nt; ++t) {
+        if (SKIP && thin(t)) {
+            __syncthreads();   // the chains' states are written by other threads here
+            const int row = tid >> 2, e = tid & 3;
+            const float nf = nfs[row];
+#pragma unroll 1
+            for (int x = 0; x < 32; ++x) {   // the tile's groups, chain by chain in order
+                const int v = grp[(t & 1) * 32 + x];
+                if (v < 0) continue;
+                const long long s = s_begin + (long long)v * 64 + (x & 15) * 4 + e;
+                const float ls = (s < s_end && !b.mask[s]) ? b.logw[s] : -INFINITY;
+                float s1, s2;
+                pair_sums_thread(b.u + (size_t)(i0 + row) * rp, b.f + (size_t)(i0 + row) * rp, b.u + (size_t)s * rp, rp, s1, s2);
+#pragma unroll
+                for (int j = 0; j < N; ++j) {
+                    const float v0 = fmaf(-s1, k.inv2tau[j], s2) + (__fmul_rn(-0.5f * k.tau[j], nf) + ls);
+                    float sc[4];
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) sc[c] = __shfl_sync(0xffffffffu, v0, (tid & 28) + c);
+                    if (e == 0) add4(lse + (size_t)((row & 3) * N + j) * 2 * THREADS + (row >> 2) * 16 + (x & 15), sc);
+                }
+            }
+            if (t + 1 < nt) next_groups(t + 1);
+            __syncthreads();
+            if (t + 1 < nt) {
+                if (!thin(t + 1)) load(t + 1, 0, buf);
+                if (tid < BN) lsrc[((t + 1) & 1) * BN + tid] = source_term(t + 1);
+            }
+            continue;
+        }
         uint64_t S1[RP][TN], S2[RP][TN];
 #pragma unroll
         for (int p = 0; p < RP; ++p)
 #pragma unroll
             for (int c = 0; c < TN; ++c) { S1[p][c] = 0ull; S2[p][c] = 0ull; }
+        bool dead = false;
         for (int c = 0; c < nch; ++c, buf ^= 1) {
             cp_wait_all();
             __syncthreads();   // the stage landed; the other buffer and the last tile are done with
             const bool last = c + 1 == nch;
             if (!last) load(t, c + 1, buf ^ 1);
-            else if (t + 1 < nt) load(t + 1, 0, buf ^ 1);
-            const float nls = (c == 0 && t + 1 < nt) ? source_term(t + 1) : 0.f;
+            else if (t + 1 < nt && !thin(t + 1)) load(t + 1, 0, buf ^ 1);
+            // the next tile's source terms (SKIP: its groups first, one stage earlier)
+            if (SKIP && c == 0 && t + 1 < nt) next_groups(t + 1);
+            const bool take = c == (SKIP ? 1 : 0) && t + 1 < nt;
+            const float nls = take ? source_term(t + 1) : 0.f;
             const float* A = st0 + buf * SW + ty * 4;
             const float* F = A + BK * AS;
             const float* M = F + BK * AS;
@@ -223,8 +433,49 @@ __device__ __forceinline__ void block(const Consts<float>& k, const Bufs<float>&
 #pragma unroll 1
                 for (int kk = 0; kk < kc; ++kk) coord(kk);
             }
-            if (c == 0 && t + 1 < nt && tid < BN) lsrc[((t + 1) & 1) * BN + tid] = nls;
+            if (take && tid < BN) lsrc[((t + 1) & 1) * BN + tid] = nls;
+            if (SKIP && (c & 3) == 3 && nch - 1 - c >= 4) {
+                // every pair of the tile already below its row's threshold at every scale?
+                float ls[TN];
+#pragma unroll
+                for (int g = 0; g < TN / 4; ++g) {
+                    const float4 lv = *reinterpret_cast<const float4*>(lsrc + (t & 1) * BN + 64 * g + tx * 4);
+                    ls[4 * g] = lv.x; ls[4 * g + 1] = lv.y; ls[4 * g + 2] = lv.z; ls[4 * g + 3] = lv.w;
+                }
+                // (a row's own term, D = 0, is known: it does not keep the tile)
+                const int own = own_group(t);
+                bool alive = false;
+#pragma unroll
+                for (int a = 0; a < TM; ++a)
+#pragma unroll
+                    for (int j = 0; j < N; ++j) {
+                        float m = -INFINITY;
+#pragma unroll
+                        for (int e = 0; e < TN; ++e)
+                            if (!((e & 3) == a && (e >> 2) == own)) m = max_nan(m, fmaf(-lane2(S1[a >> 1][e], a & 1), k.inv2tau[j], lane2(S2[a >> 1][e], a & 1)) + ls[e]);
+                        alive |= !(m < thr[(ty * 4 + a) * N + j]);
+                    }
+                if (!__syncthreads_or(alive)) {
+                    if (own >= 0) {
+#pragma unroll
+                        for (int a = 0; a < TM; ++a)
+#pragma unroll
+                            for (int j = 0; j < N; ++j) {
+                                float sc[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+                                sc[a] = 0.f + (__fmul_rn(-0.5f * k.tau[j], nfs[ty * 4 + a]) + (own ? ls[4 + a] : ls[a]));
+                                add4(lse + (size_t)(a * N + j) * 2 * THREADS + tid, sc);
+                            }
+                    }
+                    cp_wait_all();   // the stage under way is of no use
+                    __syncthreads();
+                    if (t + 1 < nt && !thin(t + 1)) load(t + 1, 0, buf ^ 1);
+                    dead = true;
+                    buf ^= 1;
+                    break;
+                }
+            }
         }
+        if (SKIP && dead) continue;
         if constexpr (OP) {
             const size_t plane = (size_t)k.n_pad * (size_t)k.n_pad;
 #pragma unroll
@@ -266,22 +517,7 @@ __device__ __forceinline__ void block(const Consts<float>& k, const Bufs<float>&
                         for (int c = 0; c < 4; ++c)
                             sc[c] = fmaf(-lane2(S1[a >> 1][4 * g + c], a & 1), k.inv2tau[j],
                                          lane2(S2[a >> 1][4 * g + c], a & 1)) + (rc + ls[c]);
-                        float tmax = max_nan(max_nan(sc[0], sc[1]), max_nan(sc[2], sc[3]));
-                        float* sp = lse + (size_t)(a * N + j) * 2 * THREADS + tid;
-                        float mx = sp[0];
-                        // every term zero in float32 (a NaN compares false and is taken in)
-                        if (tmax < mx - kZeroGap) continue;
-                        if (tmax != tmax) tmax = fmaxf(fmaxf(sc[0], sc[1]), fmaxf(sc[2], sc[3]));
-                        if (!(tmax > -INFINITY)) continue;   // no live source
-                        float sm = sp[THREADS];
-                        if (tmax > mx) {
-                            sm = (mx == -INFINITY) ? 0.f : sm * exp_hw(mx - tmax);
-                            mx = tmax;
-                        }
-#pragma unroll
-                        for (int c = 0; c < 4; ++c) sm += exp_hw(sc[c] - mx);
-                        sp[0] = mx;
-                        sp[THREADS] = sm;
+                        add4(lse + (size_t)(a * N + j) * 2 * THREADS + tid, sc);
                     }
                 }
             }

@@ -49,3 +49,37 @@ def test_prediction_at_tile_edges(yy_lib, r, n, N, noise):
     ok, kappa = combination_err_ok(got[both], ref[both], Lj[both], p.coef, lw64[both], 1e-5)
     print(f"r={r} n={n} N={N} noise={noise}: largest condition number {kappa:.1f}")
     assert ok
+
+
+@pytest.mark.parametrize("r,n,N", [(128, 300, 2), (130, 1000, 3), (200, 2049, 1), (256, 777, 4), (1000, 513, 2)])
+@pytest.mark.parametrize("spread", [0.0, 60.0, 3000.0, 1e5])
+def test_long_rows_with_spread_weights(yy_lib, r, n, N, spread):
+    """Long rows leave out terms that are zero in float32 next to the row's largest: the
+    weights of a restart, of a posterior a few thousand nats wide (whole groups of sources
+    drop out) and of the large-scale model after an update (1e5 nats), with dead and masked
+    sources among them, against the oracle, which takes every term.  A log-weight of
+    magnitude L carries its own float32 rounding, so the bar is relative to max(1, |ref|)."""
+    from oracle import filter as F
+    from paper_2509_16896_gb300 import binding
+    f = binding.Filter(binding.make_config(model="cubic", r=r, n=n, dt=0.01, R=0.3, n_scales=N, precision="f32"))
+    poly, scr = sobol_inputs(r, 50 + r)
+    f.init_nodes(poly, scr, np.zeros(r))
+    u, _ = f.get_nodes()
+    p = oracle_problem("cubic", r, n, 0.01, 0.3, N)
+    rng = np.random.default_rng(r + n + int(spread))
+    lw = (-spread * rng.random(n)).astype(np.float32)
+    lw[rng.random(n) < 0.1] = -np.inf
+    lw[n // 2] = 0.0
+    centre = rng.standard_normal(r)
+    f.set_state(centre, lw, 0.0, 1)
+    f.predict()
+    pred, off = f.get_log_weights()
+    prep = F.prepare(p, u, centre)
+    lw64 = lw.astype(np.float64)
+    Lj = F.kernel_lse(p, prep, lw64)
+    ref, _ = F.combine(p, Lj, lw64, prep.mask)
+    got = pred.astype(np.float64) + off
+    both = np.isfinite(got) == np.isfinite(ref)
+    assert both.mean() >= 0.99, np.nonzero(~both)[0][:5]
+    ok, _ = combination_err_ok(got[both], ref[both], Lj[both], p.coef, lw64[both], 1e-5)
+    assert ok
