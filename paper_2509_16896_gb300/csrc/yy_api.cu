@@ -201,9 +201,10 @@ size_t carve(const yy_config* c, char* base, Bufs<T>* out) {
         b.nu_chunk = cv.take<float>((size_t)n_pad * (r_pad / kColAlign) * sizeof(float));
     // plain form of a filter with fewer than two target blocks of 64 per SM: its source
     // ranges' partial states
-    if ((c->precision == YY_PREC_FP32 || c->precision == YY_PREC_FP64) && n_pad < 2 * kSms * 64)
+    if (c->precision != YY_PREC_BF16 && n_pad < 2 * kSms * 64)
         b.simt_part = cv.take<T>((size_t)n_pad * kSimtMaxSplit * kMaxScales * 2 * sizeof(T));
-    if (c->precision == YY_PREC_FP32 || c->precision == YY_PREC_BF16)
+    if (c->precision == YY_PREC_FP32_SCREEN) b.scr_flags = cv.take<uint32_t>(scr_flag_words(n_pad) * sizeof(uint32_t));
+    if (c->precision != YY_PREC_FP64)
         b.pair_ref = cv.take<float>((size_t)n_pad * kMaxScales * sizeof(float));
     if (c->precision == YY_PREC_BF16) {
         b.tc_q = cv.take<float>((size_t)n_pad * sizeof(float));
@@ -552,8 +553,9 @@ yy_status yy_predict(yy_filter* f) {
         const int nk = f->r_pad / kColAlign;
         const int k1 = kColAlign * (f->cfg.screen_prefix > 0 ? f->cfg.screen_prefix : (nk + 1) / 2);
         e = cudaMemsetAsync(&f->bf.stats->clamps, 0, sizeof(unsigned), f->stream);
-        if (e == cudaSuccess) e = launch_ksum_scr32(f->kf, f->bf, k1, f->stream);
-        f->launches += 2;
+        int l = 0;
+        if (e == cudaSuccess) e = launch_ksum_scr32(f->kf, f->bf, k1, f->stream, &l);
+        f->launches += l;
     } else {
         e = cudaMemsetAsync(&f->bf.stats->clamps, 0, sizeof(unsigned), f->stream);
         int l = 0;

@@ -52,7 +52,6 @@ struct DevStats {
     unsigned long long tc_last_blk, tc_last_esc;   // the same, kept for the host
     int tc_last_nk1;             // first-pass chunks the last prediction used
     unsigned int tc_done;        // CTAs of the running prediction launch that finished
-    float scr_lmax;              // screened float32 form: largest live source log-weight
     int op_stale;                // the materialised operator must be rebuilt (nodes moved)
 };
 
@@ -146,6 +145,7 @@ struct Bufs {
     float* tc_part;       // [n_pad][8][4][2] partial (max, sum) of split work items
     T* simt_part;         // [n_pad][kSimtMaxSplit][kMaxScales][2] plain forms: partial (max, sum)
                           // of each source range (filters with few target blocks only)
+    uint32_t* scr_flags;  // FP32 screen: per block of 32 targets a bit per tile of 128 sources
     float* pair_ref;      // [n_pad][kMaxScales] plain float32 form of long rows: lower bounds of the
                           // rows' largest scores
     int4* tc_items;       // single-filter work list (target tile, split, nsplit)
@@ -193,7 +193,12 @@ cudaError_t launch_prep(const Consts<T>& k, const Bufs<T>& b, bool init_weights,
 cudaError_t launch_ksum_simt(const Consts<double>& k, const Bufs<double>& b, cudaStream_t s, int* launches = nullptr);
 cudaError_t launch_pair(const Consts<float>& k, const Bufs<float>& b, cudaStream_t s, int* launches);
 cudaError_t prepare_pair();
-cudaError_t launch_ksum_scr32(const Consts<float>& k, const Bufs<float>& b, int k1, cudaStream_t s);
+bool pair_skip_fits(const Consts<float>& k, const Bufs<float>& b);
+cudaError_t launch_pair_ref(const Consts<float>& k, const Bufs<float>& b, cudaStream_t s);
+cudaError_t launch_pair_flagged(const Consts<float>& k, const Bufs<float>& b, float gap, const uint32_t* flags,
+                                int fwords, cudaStream_t s, int* launches);
+size_t scr_flag_words(long long n_pad);
+cudaError_t launch_ksum_scr32(const Consts<float>& k, const Bufs<float>& b, int k1, cudaStream_t s, int* launches);
 cudaError_t launch_op_build(const Consts<float>& k, const Bufs<float>& b, bool force, cudaStream_t s);
 cudaError_t launch_op_apply(const Consts<float>& k, const Bufs<float>& b, cudaStream_t s);
 cudaError_t prepare_op_apply();

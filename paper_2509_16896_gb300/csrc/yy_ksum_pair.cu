@@ -123,6 +123,18 @@ constexpr int kSkipMinDim = 128;
 constexpr size_t kMaxMaskBytes = 32768;   // ranges of up to a million sources
 constexpr float kSkipGap = 110.0f;
 
+// Source ranges per target row (at most kSimtMaxSplit, none beyond the source groups): two
+// blocks of 64 targets per SM where the filter has few targets and the workspace holds the
+// partial states.
+int pair_splits(const Consts<float>& k, const Bufs<float>& b, long long rows) {
+    if (!b.simt_part) return 1;
+    const long long blocks = (rows + 63) / 64;
+    long long sp = (2 * kSms + blocks - 1) / blocks;
+    sp = std::min<long long>(sp, kSimtMaxSplit);
+    sp = std::min<long long>(sp, k.n_pad / 64);
+    return (int)std::max<long long>(sp, 1);
+}
+
 template <int N>
 cudaError_t set_attr_n() {
     const auto a = cudaFuncAttributeMaxDynamicSharedMemorySize;
@@ -133,23 +145,39 @@ cudaError_t set_attr_n() {
     return e;
 }
 
+template <int N>
+cudaError_t launch_ref_n(const Consts<float>& k, const Bufs<float>& b, cudaStream_t s) {
+    const long long rows = k.row1 - k.row0;
+    k_pair_ref<N><<<(unsigned)std::min<long long>((rows + 7) / 8, 2 * kSms), 256, 0, s>>>(k, b);
+    return cudaGetLastError();
+}
+size_t mask_bytes(long long n, int S) { return 16 * sizeof(uint32_t) * (size_t)mask_words(n, S); }
+
 template <int N, bool NOISE>
-cudaError_t launch_n(const Consts<float>& k, const Bufs<float>& b, long long rows, int S, cudaStream_t s, int* l) {
-    const unsigned grid = (unsigned)((rows + BM - 1) / BM * S);
-    const size_t mask = 16 * sizeof(uint32_t) * (size_t)mask_words(k.n, S);
-    if (!NOISE && b.pair_ref && k.r >= kSkipMinDim && mask <= kMaxMaskBytes) {
-        k_pair_ref<N><<<(unsigned)std::min<long long>((rows + 7) / 8, 2 * kSms), 256, 0, s>>>(k, b);
-        k_pair_skip<N><<<grid, THREADS, smem_bytes<N, false, false, true>() + mask, s>>>(k, b, S, kSkipGap, nullptr, 0);
+cudaError_t merge_n(const Consts<float>& k, const Bufs<float>& b, int S, cudaStream_t s) {
+    if (S > 1) k_pair_merge<N, NOISE><<<(unsigned)((k.row1 - k.row0 + 127) / 128), 128, 0, s>>>(k, b, S);
+    return cudaGetLastError();
+}
+template <int N>
+cudaError_t launch_skip_n(const Consts<float>& k, const Bufs<float>& b, int S, float gap, const uint32_t* flags,
+                          int fwords, cudaStream_t s) {
+    const unsigned grid = (unsigned)((k.row1 - k.row0 + BM - 1) / BM * S);
+    k_pair_skip<N><<<grid, THREADS, smem_bytes<N, false, false, true>() + mask_bytes(k.n, S), s>>>(k, b, S, gap, flags,
+                                                                                                  fwords);
+    const cudaError_t e = cudaGetLastError();
+    return e == cudaSuccess ? merge_n<N, false>(k, b, S, s) : e;
+}
+template <int N, bool NOISE>
+cudaError_t launch_n(const Consts<float>& k, const Bufs<float>& b, int S, cudaStream_t s, int* l) {
+    if (!NOISE && k.r >= kSkipMinDim && pair_skip_fits(k, b)) {
         if (l) *l += 1;
-    } else {
-        k_pair<N, NOISE><<<grid, THREADS, smem_bytes<N, NOISE, false>(), s>>>(k, b, S);
+        const cudaError_t e = launch_ref_n<N>(k, b, s);
+        return e == cudaSuccess ? launch_skip_n<N>(k, b, S, kSkipGap, nullptr, 0, s) : e;
     }
-    cudaError_t e = cudaGetLastError();
-    if (e == cudaSuccess && S > 1) {
-        k_pair_merge<N, NOISE><<<(unsigned)((rows + 127) / 128), 128, 0, s>>>(k, b, S);
-        e = cudaGetLastError();
-    }
-    return e;
+    const unsigned grid = (unsigned)((k.row1 - k.row0 + BM - 1) / BM * S);
+    k_pair<N, NOISE><<<grid, THREADS, smem_bytes<N, NOISE, false>(), s>>>(k, b, S);
+    const cudaError_t e = cudaGetLastError();
+    return e == cudaSuccess ? merge_n<N, NOISE>(k, b, S, s) : e;
 }
 
 }  // namespace
@@ -164,18 +192,6 @@ cudaError_t prepare_pair() {
     return e;
 }
 
-// Source ranges per target row (at most kSimtMaxSplit, none beyond the source groups): two
-// blocks of 64 targets per SM where the filter has few targets and the workspace holds the
-// partial states.
-static int pair_splits(const Consts<float>& k, const Bufs<float>& b, long long rows) {
-    if (!b.simt_part) return 1;
-    const long long blocks = (rows + 63) / 64;
-    long long sp = (2 * kSms + blocks - 1) / blocks;
-    sp = std::min<long long>(sp, kSimtMaxSplit);
-    sp = std::min<long long>(sp, k.n_pad / 64);
-    return (int)std::max<long long>(sp, 1);
-}
-
 cudaError_t launch_pair(const Consts<float>& k, const Bufs<float>& b, cudaStream_t s, int* launches) {
     const long long rows = k.row1 - k.row0;
     if (rows <= 0) return cudaSuccess;
@@ -183,10 +199,41 @@ cudaError_t launch_pair(const Consts<float>& k, const Bufs<float>& b, cudaStream
     const bool noise = k.noise == YY_NOISE_DIAG;
     if (launches) *launches += S > 1 ? 2 : 1;
     switch (k.N) {
-        case 1: return noise ? launch_n<1, true>(k, b, rows, S, s, launches) : launch_n<1, false>(k, b, rows, S, s, launches);
-        case 2: return noise ? launch_n<2, true>(k, b, rows, S, s, launches) : launch_n<2, false>(k, b, rows, S, s, launches);
-        case 3: return noise ? launch_n<3, true>(k, b, rows, S, s, launches) : launch_n<3, false>(k, b, rows, S, s, launches);
-        case 4: return noise ? launch_n<4, true>(k, b, rows, S, s, launches) : launch_n<4, false>(k, b, rows, S, s, launches);
+        case 1: return noise ? launch_n<1, true>(k, b, S, s, launches) : launch_n<1, false>(k, b, S, s, launches);
+        case 2: return noise ? launch_n<2, true>(k, b, S, s, launches) : launch_n<2, false>(k, b, S, s, launches);
+        case 3: return noise ? launch_n<3, true>(k, b, S, s, launches) : launch_n<3, false>(k, b, S, s, launches);
+        case 4: return noise ? launch_n<4, true>(k, b, S, s, launches) : launch_n<4, false>(k, b, S, s, launches);
+    }
+    return cudaErrorInvalidValue;
+}
+
+// The masks of a source range fit the skipping form's shared memory.
+bool pair_skip_fits(const Consts<float>& k, const Bufs<float>& b) {
+    return b.pair_ref && mask_bytes(k.n, pair_splits(k, b, k.row1 - k.row0)) <= kMaxMaskBytes;
+}
+
+cudaError_t launch_pair_ref(const Consts<float>& k, const Bufs<float>& b, cudaStream_t s) {
+    if (k.row1 <= k.row0) return cudaSuccess;
+    switch (k.N) {
+        case 1: return launch_ref_n<1>(k, b, s);
+        case 2: return launch_ref_n<2>(k, b, s);
+        case 3: return launch_ref_n<3>(k, b, s);
+        case 4: return launch_ref_n<4>(k, b, s);
+    }
+    return cudaErrorInvalidValue;
+}
+
+cudaError_t launch_pair_flagged(const Consts<float>& k, const Bufs<float>& b, float gap, const uint32_t* flags,
+                                int fwords, cudaStream_t s, int* launches) {
+    const long long rows = k.row1 - k.row0;
+    if (rows <= 0) return cudaSuccess;
+    const int S = pair_splits(k, b, rows);
+    if (launches) *launches += S > 1 ? 2 : 1;
+    switch (k.N) {
+        case 1: return launch_skip_n<1>(k, b, S, gap, flags, fwords, s);
+        case 2: return launch_skip_n<2>(k, b, S, gap, flags, fwords, s);
+        case 3: return launch_skip_n<3>(k, b, S, gap, flags, fwords, s);
+        case 4: return launch_skip_n<4>(k, b, S, gap, flags, fwords, s);
     }
     return cudaErrorInvalidValue;
 }

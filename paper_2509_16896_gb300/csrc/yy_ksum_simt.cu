@@ -1,6 +1,6 @@
 // Prediction step on the FMA pipes: the plain form in float64 (and in float32 for batches),
-// the screened float32 form and the materialised operator's apply.  The plain float32 form of a
-// single filter is in yy_ksum_pair.cu.
+// and the materialised operator's apply.  The plain float32 form of a single filter is in
+// yy_ksum_pair.cu, the screened one in yy_ksum_scr.cu.
 //
 // For every target i and scale j (tau_j = dt / 2^(j-1)), in units relative to c_ref:
 //   L_j(i) - c_ref = (C_j - c_ref) - tau_j div f(x_i)
@@ -35,31 +35,15 @@ template <> __device__ __forceinline__ float exp_fast<float>(float x) { return e
 template <> __device__ __forceinline__ double exp_fast<double>(double x) { return exp(x); }
 }  // namespace
 
-// SCREEN (float32 only): before a source tile is evaluated, the squared distance of each
-// of its pairs over the first k1 coordinates -- a lower bound of the full |u_i - u_s|^2 --
-// is bounded from below through its Gram form q_i + q_s - 2 G (q the norms over those
-// coordinates from the preparation pass, G = sum u_i u_s by one FMA per coordinate), less
-// the rounding allowance 3 gamma_k1 (q_i + q_s) of the FMA chain (gamma_k = k 2^-24 /
-// (1 - k 2^-24); 2 |u_i||u_s| <= q_i + q_s) and 1e-5 (q_i + q_s) for the norms' own
-// rounding, and compared with rho_i^2, where
-//     rho_i = max_j [tau_j |f_i| + sqrt(2 tau_j max(0, lmax - (ell_i - tau_j |f_i|^2 / 2) + T))],
-// lmax the largest live source log-weight, ell_i - tau_j |f_i|^2 / 2 the exact self term of
-// row i (a lower bound of its largest term) and T = ln n + 20.  By the triangle inequality
-// |u_i - tau_j f_i - u_s| >= |u_i - u_s| - tau_j |f_i|, a pair beyond rho_i scores below the
-// self term by more than T at every scale, so a tile none of whose live pairs passes is
-// skipped (all skipped terms together are below e^-20 of the row's sum); any other tile is
-// evaluated exactly as in the plain form.  A live target without a finite log-weight has no
-// reference and takes every tile.  The comparison carries a relative margin of 1e-4 for
-// the float32 rounding of the partial sums.
 // NOISE (diagonal noise coefficients): the squared distance and the drift's inner product
 // take the target's metric a(x_i)^+, S1 = sum_d m_d D_d^2, S2 = sum_d m_d D_d f_d, with
 // |f_i|^2 in the same metric (nf) and -1/2 log det_+ a(x_i) added in the combination.
 // split / nsplit (plain form of a filter with few target blocks): this block sweeps only the
 // split-th of nsplit equal ranges of source tiles and stores its rows' partial (max, sum)
 // per scale in b.simt_part; k_simt_merge combines the ranges.
-template <typename T, int N, bool SCREEN = false, bool NOISE = false>
-__device__ __forceinline__ void ksum_simt_body(const Consts<T>& k, const Bufs<T>& b, int rk, int bid, int k1 = 0,
-                                               int split = 0, int nsplit = 1) {
+template <typename T, int N, bool NOISE = false>
+__device__ __forceinline__ void ksum_simt_body(const Consts<T>& k, const Bufs<T>& b, int rk, int bid, int split = 0,
+                                               int nsplit = 1) {
     __shared__ T At[BK][BM];   // u of targets
     __shared__ T Ft[BK][BM];   // f of targets
     __shared__ T Bt[BK][BN];   // u of sources
@@ -72,10 +56,6 @@ __device__ __forceinline__ void ksum_simt_body(const Consts<T>& k, const Bufs<T>
 
     T rowc[TM][N];          // -(tau_j / 2) |f_i|^2
     T mx[TM][N], sm[TM][N];
-    T rho2[TM];             // SCREEN: squared screening radius of each row
-    T q1t[TM];              // SCREEN: first-pass norms of the target rows
-    __shared__ T q1s[SCREEN ? BN : 1];   // SCREEN: first-pass norms of the tile's sources
-    const T gam = SCREEN ? T(3.03) * (T)k1 * T(5.9604645e-8) + T(1e-5) : T(0);   // rounding allowance per (q_i + q_s)
 #pragma unroll
     for (int a = 0; a < TM; ++a) {
         const long long i = i0 + ty * TM + a;
@@ -85,31 +65,6 @@ __device__ __forceinline__ void ksum_simt_body(const Consts<T>& k, const Bufs<T>
             rowc[a][j] = -T(0.5) * k.tau[j] * nf;
             mx[a][j] = T(-INFINITY);
             sm[a][j] = T(0);
-        }
-        rho2[a] = T(-1);   // no candidates (padded or masked rows)
-        if constexpr (SCREEN) {   // first-pass norm of the target row
-            q1t[a] = T(0);
-            if (i < k.n)
-                for (int c = 0; c < k1 / 64; ++c) q1t[a] += b.nu_chunk[(size_t)i * (k.r_pad / 64) + c];
-        }
-        if constexpr (SCREEN) {
-            if (i < k.n && !b.mask[i]) {
-                const T li = b.logw[i];
-                const T lmax = (T)b.stats->scr_lmax;
-                if (li == T(-INFINITY)) {
-                    rho2[a] = T(INFINITY);
-                } else {
-                    const T Tn = log((T)k.n) + T(20);
-                    const T Fi = sqrt(nf);
-                    T rho = T(0);
-#pragma unroll
-                    for (int j = 0; j < N; ++j) {
-                        const T gap = fmax(lmax - (rowc[a][j] + li) + Tn, T(0));
-                        rho = fmax(rho, k.tau[j] * Fi + sqrt(T(2) * k.tau[j] * gap));
-                    }
-                    rho2[a] = rho * rho * T(1.0001) + T(1e-30);
-                }
-            }
         }
     }
 
@@ -125,52 +80,6 @@ __device__ __forceinline__ void ksum_simt_body(const Consts<T>& k, const Bufs<T>
         if (tid < BN) {
             const long long s = s0 + tid;
             lsrc[tid] = (s < k.n && !b.mask[s]) ? b.logw[s] : T(-INFINITY);
-            if constexpr (SCREEN) {
-                T q = T(0);
-                if (s < k.n)
-                    for (int c = 0; c < k1 / 64; ++c) q += b.nu_chunk[(size_t)s * (k.r_pad / 64) + c];
-                q1s[tid] = q;
-            }
-        }
-        if constexpr (SCREEN) {
-            // first pass: Gram products G over coordinates [0, k1)
-            for (int d0 = 0; d0 < k1; d0 += BK) {
-                __syncthreads();
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const int e = tid + 256 * q;
-                    const int row = e >> 4, col = e & 15;
-                    At[col][row] = (T)b.u[(size_t)(i0 + row) * k.r_pad + d0 + col];
-                    Bt[col][row] = (T)b.u[(size_t)(s0 + row) * k.r_pad + d0 + col];
-                }
-                __syncthreads();
-#pragma unroll
-                for (int kk = 0; kk < BK; ++kk) {
-                    T av[TM], bv[TN];
-#pragma unroll
-                    for (int a = 0; a < TM; ++a) av[a] = At[kk][ty * TM + a];
-#pragma unroll
-                    for (int c = 0; c < TN; ++c) bv[c] = Bt[kk][tx * TN + c];
-#pragma unroll
-                    for (int a = 0; a < TM; ++a)
-#pragma unroll
-                        for (int c = 0; c < TN; ++c) S1[a][c] = fma(av[a], bv[c], S1[a][c]);
-                }
-            }
-            int any = 0;
-#pragma unroll
-            for (int a = 0; a < TM; ++a)
-#pragma unroll
-                for (int c = 0; c < TN; ++c) {
-                    const T qq = q1t[a] + q1s[tx * TN + c];
-                    const T lower = qq - T(2) * S1[a][c] - gam * qq;   // lower bound of the partial |u_i - u_s|^2
-                    any |= (lower <= rho2[a] && lsrc[tx * TN + c] != T(-INFINITY)) ? 1 : 0;
-                }
-            if (!__syncthreads_or(any)) continue;   // every pair of the tile is negligible
-#pragma unroll
-            for (int a = 0; a < TM; ++a)
-#pragma unroll
-                for (int c = 0; c < TN; ++c) S1[a][c] = T(0);
         }
         for (int d0 = 0; d0 < rk; d0 += BK) {
             __syncthreads();
@@ -282,7 +191,7 @@ __device__ __forceinline__ void ksum_simt_body(const Consts<T>& k, const Bufs<T>
 
 template <typename T, int N, bool NOISE = false>
 __global__ void __launch_bounds__(256) k_ksum_simt(Consts<T> k, Bufs<T> b, int rk, int nsplit) {
-    ksum_simt_body<T, N, false, NOISE>(k, b, rk, (int)(k.row0 / BM) + (int)(blockIdx.x / nsplit), 0,
+    ksum_simt_body<T, N, NOISE>(k, b, rk, (int)(k.row0 / BM) + (int)(blockIdx.x / nsplit),
                                        (int)(blockIdx.x % nsplit), nsplit);
 }
 
@@ -310,11 +219,6 @@ __global__ void __launch_bounds__(256) k_simt_merge(Consts<T> k, Bufs<T> b, int 
     }
     const T hld = NOISE ? b.hld[i] : T(0);
     b.logw_pred[i] = combine_scales<T, N>(k, mx, sm, b.divf[i], b.logw[i], b.stats->c_ref, &b.stats->clamps, hld);
-}
-
-template <int N>
-__global__ void __launch_bounds__(256) k_ksum_scr32(Consts<float> k, Bufs<float> b, int rk, int k1) {
-    ksum_simt_body<float, N, true>(k, b, rk, (int)(k.row0 / BM) + blockIdx.x, k1);
 }
 
 // The apply works in base 2: with v = A + ell, e^(v - m) = 2^(v log2 e - m log2 e).
@@ -557,44 +461,6 @@ cudaError_t launch_op_apply(const Consts<float>& k, const Bufs<float>& b, cudaSt
         case 2: k_op_apply<2><<<grid, 288, op_smem_bytes<2>(), s>>>(k, b); break;
         case 3: k_op_apply<3><<<grid, 288, op_smem_bytes<3>(), s>>>(k, b); break;
         default: k_op_apply<4><<<grid, 288, op_smem_bytes<4>(), s>>>(k, b); break;
-    }
-    return cudaGetLastError();
-}
-
-// Largest live source log-weight (the screen's lmax), one block.
-__global__ void __launch_bounds__(1024) k_live_lmax(Consts<float> k, Bufs<float> b) {
-    __shared__ float red[32];
-    float m = -INFINITY;
-    for (long long i = threadIdx.x; i < k.n; i += blockDim.x)
-        if (!b.mask[i]) m = fmaxf(m, b.logw[i]);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int w = 1; w < (int)(blockDim.x >> 5); ++w) m = fmaxf(m, red[w]);
-        b.stats->scr_lmax = m;
-    }
-}
-
-// Screened float32 form: first pass over k1 coordinates (a multiple of 64, 64 <= k1 <= r
-// rounded up to 64: the first-pass norms come in chunks of 64), then exact evaluation of
-// every tile that keeps a candidate.
-cudaError_t launch_ksum_scr32(const Consts<float>& k, const Bufs<float>& b, int k1, cudaStream_t s) {
-    if (!b.nu_chunk) return cudaErrorInvalidValue;
-    const int rk = ((k.r + BK - 1) / BK) * BK;
-    k1 = ((k1 + 63) / 64) * 64;
-    if (k1 < 64) k1 = 64;
-    if (k1 > k.r_pad) k1 = k.r_pad;
-    const unsigned grid = (unsigned)((k.row1 - k.row0 + BM - 1) / BM);   // the handle's target blocks
-    if (grid == 0) return cudaSuccess;
-    k_live_lmax<<<1, 1024, 0, s>>>(k, b);
-    switch (k.N) {
-        case 1: k_ksum_scr32<1><<<grid, 256, 0, s>>>(k, b, rk, k1); break;
-        case 2: k_ksum_scr32<2><<<grid, 256, 0, s>>>(k, b, rk, k1); break;
-        case 3: k_ksum_scr32<3><<<grid, 256, 0, s>>>(k, b, rk, k1); break;
-        case 4: k_ksum_scr32<4><<<grid, 256, 0, s>>>(k, b, rk, k1); break;
-        default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
 }

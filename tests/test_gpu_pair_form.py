@@ -53,15 +53,17 @@ def test_prediction_at_tile_edges(yy_lib, r, n, N, noise):
 
 @pytest.mark.parametrize("r,n,N", [(128, 300, 2), (130, 1000, 3), (200, 2049, 1), (256, 777, 4), (1000, 513, 2)])
 @pytest.mark.parametrize("spread", [0.0, 60.0, 3000.0, 1e5])
-def test_long_rows_with_spread_weights(yy_lib, r, n, N, spread):
+@pytest.mark.parametrize("prec", ["f32", "f32s"])
+def test_long_rows_with_spread_weights(yy_lib, prec, r, n, N, spread):
     """Long rows leave out terms that are zero in float32 next to the row's largest: the
     weights of a restart, of a posterior a few thousand nats wide (whole groups of sources
     drop out) and of the large-scale model after an update (1e5 nats), with dead and masked
-    sources among them, against the oracle, which takes every term.  A log-weight of
+    sources among them, in the plain form and behind the float32 screen (terms below
+    e^-(ln n + 20)), against the oracle, which takes every term.  A log-weight of
     magnitude L carries its own float32 rounding, so the bar is relative to max(1, |ref|)."""
     from oracle import filter as F
     from paper_2509_16896_gb300 import binding
-    f = binding.Filter(binding.make_config(model="cubic", r=r, n=n, dt=0.01, R=0.3, n_scales=N, precision="f32"))
+    f = binding.Filter(binding.make_config(model="cubic", r=r, n=n, dt=0.01, R=0.3, n_scales=N, precision=prec))
     poly, scr = sobol_inputs(r, 50 + r)
     f.init_nodes(poly, scr, np.zeros(r))
     u, _ = f.get_nodes()
