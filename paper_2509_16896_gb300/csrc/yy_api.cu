@@ -535,7 +535,9 @@ yy_status yy_predict(yy_filter* f) {
     if (f->fp64) {
         e = cudaMemsetAsync(&f->bd.stats->clamps, 0, sizeof(unsigned), f->stream);
         int l = 0;
-        if (e == cudaSuccess) e = launch_ksum_simt(f->kd, f->bd, f->stream, &l);
+        if (e == cudaSuccess)
+            e = ksum_f64_fits(f->kd) ? launch_ksum_f64(f->kd, f->bd, f->stream, &l)
+                                     : launch_ksum_simt(f->kd, f->bd, f->stream, &l);
         f->launches += l;
     } else if (f->use_op) {
         // materialised schedule: rebuild on the device if the node set moved, then apply

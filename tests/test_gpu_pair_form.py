@@ -85,3 +85,35 @@ def test_long_rows_with_spread_weights(yy_lib, prec, r, n, N, spread):
     assert both.mean() >= 0.99, np.nonzero(~both)[0][:5]
     ok, _ = combination_err_ok(got[both], ref[both], Lj[both], p.coef, lw64[both], 1e-5)
     assert ok
+
+
+@pytest.mark.parametrize("r,n,N,R", [(1, 2, 1, 2.0), (1, 300, 4, 5.0), (2, 1024, 2, 4.0), (3, 33, 2, 1.0), (8, 257, 3, 1.0),
+                                     (23, 255, 2, 0.3), (47, 129, 2, 0.3), (63, 500, 3, 0.3), (64, 321, 1, 0.3)])
+@pytest.mark.parametrize("spread", [2.0, 200.0])
+def test_float64_short_rows(yy_lib, r, n, N, R, spread):
+    """The float64 form that picks its pairs in float32: against the oracle at the edges of its
+    source tiles and row blocks, narrow and wide weights, dead sources among them, within the
+    float64 bar (1e-10 relative plus the combination's condition number)."""
+    from oracle import filter as F
+    from paper_2509_16896_gb300 import binding
+    f = binding.Filter(binding.make_config(model="cubic", r=r, n=n, dt=0.01, R=R, n_scales=N, precision="f64"))
+    poly, scr = sobol_inputs(r, 60 + r)
+    f.init_nodes(poly, scr, np.zeros(r))
+    u, _ = f.get_nodes()
+    p = oracle_problem("cubic", r, n, 0.01, R, N)
+    rng = np.random.default_rng(100 * r + n)
+    lw = -spread * rng.random(n)
+    lw[rng.random(n) < 0.05] = -np.inf
+    lw[0] = 0.0
+    centre = rng.standard_normal(r)
+    f.set_state(centre, lw, 0.0, 1)
+    f.predict()
+    pred, off = f.get_log_weights()
+    prep = F.prepare(p, u, centre)
+    Lj = F.kernel_lse(p, prep, lw)
+    ref, _ = F.combine(p, Lj, lw, prep.mask)
+    got = pred + off
+    both = np.isfinite(got) == np.isfinite(ref)
+    assert both.mean() >= 0.99, np.nonzero(~both)[0][:5]
+    ok, _ = combination_err_ok(got[both], ref[both], Lj[both], p.coef, lw[both], 1e-10, eps=2.0 ** -53)
+    assert ok
