@@ -17,8 +17,8 @@
 //  2. |c_i|^2 + |c_s|^2 - 2 G is the squared distance of the rows' rounded copies c (the products of
 //     copies are exact; 2^-9 |c_i||c_s| covers their accumulation, plus float32 rounding), and
 //     |u_i - u_s| >= |c_i - c_s| - 2 E with E the largest distance of a node from its copy, measured
-//     when the copies are made (e4m3 at r = 1000: at most 0.031 |u| over 4000 box points; the
-//     format's unit roundoff alone gives 0.14 |u_i||u_s| on G).  Tested per 32 columns
+//     when the copies are made (e4m3 at r = 1000: 0.026 |u|; a bound from the format's unit roundoff
+//     alone, 0.14 |u_i||u_s| on G, kept ten times the exact pairs there).  Tested per 32 columns
 //     first through the largest accumulator and the smallest |c_s|^2, then per column;
 //  3. by the triangle inequality |u_i - tau f_i - u_s| >= |u_i - u_s| - tau |f_i|, a pair
 //     whose distance exceeds rho_i = max_j [tau_j |f_i| + sqrt(2 tau_j max(0, lmax - M_j(i)

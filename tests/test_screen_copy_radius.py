@@ -27,7 +27,7 @@ def test_distance_of_copies_bounds_distance(kind, r, R):
         q = (cc ** 2).sum(1)
         c32 = cc.astype(np.float32)
         g = np.zeros((n, n), dtype=np.float32)
-        for d in range(min(k, r)):                             # one float32 rounding per product added
+        for d in range(k):                             # one float32 rounding per product added
             g += c32[:, d:d + 1] * c32[None, :, d]
         err = np.abs(q[:, None] + q[None] - 2.0 * g - dc ** 2)
         assert np.all(err <= 2.0 * 1.1 * 2.0 ** -9 * np.sqrt(q[:, None] * q[None]) + 2e-6 * (q[:, None] + q[None]))
