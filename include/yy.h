@@ -107,9 +107,9 @@ typedef enum { YY_RESTART_INIT_GAUSS = 0, YY_RESTART_INIT_UNIFORM = 1 } yy_resta
 typedef enum { YY_RESTART_PLAIN = 0, YY_RESTART_LEARNED = 1 } yy_restart_rule;
 
 /* Operands of the screening Gram product of the BF16 prediction (library design, not in the
- * paper): BF16 copies of the coordinates, or FP8 e4m3 copies scaled by a power of two (twice the
- * tensor rate, half the operand bytes, first-pass chunks of 128 coordinates, a larger
- * distance between a node and its copy, which the screen's bound takes in). */
+ * paper): BF16 (error bound 2^-6 |u_i||u_s|), or FP8 e4m3 with the coordinates scaled by a
+ * power of two (bound 0.135 |u_i||u_s| plus a term for subnormal coordinates; twice the
+ * tensor rate, half the operand bytes, first-pass chunks of 128 coordinates). */
 typedef enum { YY_SCREEN_BF16 = 0, YY_SCREEN_FP8 = 1 } yy_screen_type;
 
 /* Noise coefficients (Section "General Nonlinear Filtering with Noise Coefficients"):

@@ -276,24 +276,32 @@ void fill_consts(yy_filter* f, Consts<T>* k, const double* halfwidth) {
     // symmetric blocks need the long-row epilogue (r > 64)
     k->tc_sym = (c.precision == YY_PREC_BF16 && c.r > 64) ? 1 : 0;
     k->tc_split_len = 64;
-    // Screen operands: BF16 copies of u, or e4m3 copies of s u, s the largest power of two with
-    // s 8 max R <= 448 (a learned box is at most 8 times wider).  The screen measures distances
-    // between the copies, whose own distance from the nodes the preparation pass measures
-    // (tc_emax); the products of the copies are exact, and 2^-9 of |u_i||u_s| (with 10 % slack)
-    // covers their accumulation in the tensor core.
+    // Screen operands.  BF16: |dG| <= 2^-6 |u_i||u_s| (unit roundoff 2^-9 per operand, 4x
+    // slack).  FP8 e4m3 of s u, s the largest power of two with s 8 max R <= 448 (a learned
+    // box is at most 8 times wider): per product (2 2^-4 + 2^-8) |a b| = 0.129 |a b|, plus
+    // at most 2^-9 for reduced-precision accumulation inside one instruction (bound 0.14), and
+    // for subnormal codes an absolute error delta = 2^-10 / s per coordinate, which adds
+    // 1.07 delta sqrt(K) (|a| + |b|) + K delta^2 to |dG| (K coordinates); the d^2 bound is
+    // twice these, with 10 % slack.
     k->tc_fp8 = (c.precision == YY_PREC_BF16 && c.screen_type == YY_SCREEN_FP8) ? 1 : 0;
     k->tc_r8 = (int)((f->r_pad + 127) / 128 * 128);
     k->tc_s = 1.f;
     k->tc_g2 = -2.f;
-    k->tc_eps = 1.1f * 0.001953125f;
+    k->tc_eps = 0.015625f;
+    k->tc_dabs = 0.f;
+    k->tc_dabs2 = 0.f;
     if (k->tc_fp8) {
         double rmax = 0.0;
         for (int d = 0; d < c.r; ++d) rmax = fmax(rmax, halfwidth ? halfwidth[d] : c.R);
         double s = 1.0;
         while (s * 8.0 * rmax * 2.0 <= 448.0 && s < 1048576.0) s *= 2.0;
         while (s * 8.0 * rmax > 448.0 && s > 1.0 / 1048576.0) s *= 0.5;
+        const double K = (double)k->tc_r8, delta = ldexp(1.0, -10) / s;
         k->tc_s = (float)s;
         k->tc_g2 = (float)(-2.0 / (s * s));
+        k->tc_eps = 0.14f;
+        k->tc_dabs = (float)(1.1 * 2.0 * 1.07 * delta * sqrt(K));
+        k->tc_dabs2 = (float)(1.1 * 2.0 * K * delta * delta);
     }
     k->dt = (T)c.dt;
     double log_vol = 0.0;
@@ -413,7 +421,6 @@ yy_status do_init_nodes(yy_filter* f, Bufs<T>& b, Consts<T>& k, const uint32_t* 
             return YY_ERR_CUDA;
     }
     f->node_kind = node_kind;
-    if (b.ubf && (e = cudaMemsetAsync(&b.stats->tc_emax, 0, sizeof(float), s)) != cudaSuccess) return YY_ERR_CUDA;
     if ((e = launch_prep<T>(k, b, true, true, c.prior_mean, c.prior_var, s)) != cudaSuccess) return YY_ERR_CUDA;
     int l = 0;
     if ((e = launch_normalise_only<T>(k, b, s, &l)) != cudaSuccess) return YY_ERR_CUDA;

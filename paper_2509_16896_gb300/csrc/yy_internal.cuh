@@ -52,7 +52,6 @@ struct DevStats {
     unsigned long long tc_last_blk, tc_last_esc;   // the same, kept for the host
     int tc_last_nk1;             // first-pass chunks the last prediction used
     unsigned int tc_done;        // CTAs of the running prediction launch that finished
-    float tc_emax;               // tensor-core screen: largest |u_i - copy of u_i| of the node set
     int op_stale;                // the materialised operator must be rebuilt (nodes moved)
 };
 
@@ -75,7 +74,9 @@ struct Consts {
     int tc_r8;               // FP8: coordinates per row of the e4m3 copy (multiple of 128)
     float tc_s;              // FP8: power-of-two scale of the coordinates in the e4m3 copy
     float tc_g2;             // factor turning the accumulator into -2 G (-2, or -2 / s^2)
-    float tc_eps;            // relative error bound of the tensor core's sums per |u_i||u_s|
+    float tc_eps;            // relative error bound of G per |u_i||u_s|
+    float tc_dabs;           // FP8: absolute error term per (|u_i| + |u_s|) (subnormal codes)
+    float tc_dabs2;          // FP8: constant error term
     T logabs_c[kMaxScales + 1];
     T sign_c[kMaxScales + 1];  // 0 for a zero coefficient
     double c_ref;

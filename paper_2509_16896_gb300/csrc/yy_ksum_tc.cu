@@ -14,12 +14,11 @@
 //     MMA of source tile t+1 overlaps the screening of tile t), first over a prefix of the
 //     coordinates (a lower bound of the distance), the tiles that keep candidates again
 //     over all of them;
-//  2. |c_i|^2 + |c_s|^2 - 2 G is the squared distance of the rows' rounded copies c (the products of
-//     copies are exact; 2^-9 |c_i||c_s| covers their accumulation, plus float32 rounding), and
-//     |u_i - u_s| >= |c_i - c_s| - 2 E with E the largest distance of a node from its copy, measured
-//     when the copies are made (e4m3 at r = 1000: 0.026 |u|; a bound from the format's unit roundoff
-//     alone, 0.14 |u_i||u_s| on G, kept ten times the exact pairs there).  Tested per 32 columns
-//     first through the largest accumulator and the smallest |c_s|^2, then per column;
+//  2. |u_i - u_s|^2 ~= |u_i|^2 + |u_s|^2 - 2 G with a rigorous error bound
+//     (|dG| <= 2^-6 |u_i||u_s| for BF16 operands with FP32 accumulation; for e4m3
+//     0.14 |u_i||u_s| + 1.07 delta sqrt(K) (|u_i| + |u_s|) + K delta^2, delta = 2^-10 / s;
+//     plus float32 rounding), tested per 32 columns first through the largest accumulator
+//     and the smallest |u_s|^2, then per column;
 //  3. by the triangle inequality |u_i - tau f_i - u_s| >= |u_i - u_s| - tau |f_i|, a pair
 //     whose distance exceeds rho_i = max_j [tau_j |f_i| + sqrt(2 tau_j max(0, lmax - M_j(i)
 //     + T))] has score_j < M_j(i) - T for every scale, where M_j(i) is the running maximum
@@ -171,12 +170,12 @@ __device__ __forceinline__ float sqrt_up(float x) {
     return x > 0.f ? x * rsqrtf(x) * 1.000001f : 0.f;
 }
 
-// Screening threshold on |u_s|^2 - 2 G for one target row (see the file comment).  e2: twice the
-// largest distance of a node from its copy (copy_radius2).  rnu_i and rnumax are the square roots of nu_i and numax (per row and per tile, precomputed).
+// Screening threshold on |u_s|^2 - 2 G for one target row (see the file comment).  rnu_i
+// and rnumax are the square roots of nu_i and numax (per row and per tile, precomputed).
 template <int N>
 __device__ __forceinline__ float screen_theta(const Consts<float>& k, bool live, float nu_i, float rnu_i, float Fi,
                                               const float (&mx)[N], float lmax, float numax, float rnumax,
-                                              float T, float e2) {
+                                              float T) {
     if (!live || lmax == -INFINITY) return -INFINITY;
     float rho = 0.f;
 #pragma unroll
@@ -185,12 +184,10 @@ __device__ __forceinline__ float screen_theta(const Consts<float>& k, bool live,
         const float gap = fmaxf(lmax - mx[j] + T, 0.f);
         rho = fmaxf(rho, k.tau[j] * Fi + sqrt_up(2.f * k.tau[j] * gap));
     }
-    rho += e2;
-    const float err = 2.f * k.tc_eps * rnu_i * rnumax + 2e-6f * (nu_i + numax + rho * rho);
+    const float err = 2.f * k.tc_eps * rnu_i * rnumax + k.tc_dabs * (rnu_i + rnumax) + k.tc_dabs2 +
+                      2e-6f * (nu_i + numax + rho * rho);
     return fminf(rho * rho + err - nu_i, tc::kThetaMax);
 }
-
-__device__ __forceinline__ float copy_radius2(const DevStats* st) { return 2.00001f * st->tc_emax; }
 
 }  // namespace
 
@@ -441,9 +438,10 @@ __device__ __forceinline__ void colprep2_body(const Consts<float>& k, const Bufs
                 rho = fmaxf(rho, k.tau[j] * Fc + sqrtf(2.f * k.tau[j] * gap));
             }
             const float q = b.nu[c], q1 = b.tc_q1t[c];
-            rho += copy_radius2(b.stats);
-            const float e = 2.f * k.tc_eps * sqrtf(q * ng) + 2e-6f * (q + ng + rho * rho);
-            const float e1 = 2.f * k.tc_eps * sqrtf(q1 * ng1) + 2e-6f * (q1 + ng1 + rho * rho);
+            const float e = 2.f * k.tc_eps * sqrtf(q * ng) + k.tc_dabs * (sqrtf(q) + sqrtf(ng)) + k.tc_dabs2 +
+                            1e-6f * (q + ng + rho * rho);
+            const float e1 = 2.f * k.tc_eps * sqrtf(q1 * ng1) + k.tc_dabs * (sqrtf(q1) + sqrtf(ng1)) + k.tc_dabs2 +
+                             1e-6f * (q1 + ng1 + rho * rho);
             qt = q - fminf(rho * rho + e, tc::kThetaMax);
             qt1 = q1 - fminf(rho * rho + e1, tc::kThetaMax);
         }
@@ -857,7 +855,6 @@ __global__ void __launch_bounds__(tc::NUM_THREADS, 1)
             const Bufs<float>& b = *bp;
             const bool pre = nk1 < nk;
             const float T = logf((float)k.n) + 20.0f;
-            const float e2 = copy_radius2(b.stats);
             const long long i = i0 + q * 32 + lane;
             const bool in_range = i < k.n;
             const bool live = in_range && !b.mask[i];
@@ -1046,7 +1043,7 @@ __global__ void __launch_bounds__(tc::NUM_THREADS, 1)
                         numax = fmaxf(numax, first_pass ? ci[10] : ci[9]);
                         rnumax = fmaxf(rnumax, first_pass ? ci[14] : ci[13]);
                     }
-                    return screen_theta<N>(k, live, nu_s, rnu_s, Fi, mx, lmax, numax, rnumax, T, e2);
+                    return screen_theta<N>(k, live, nu_s, rnu_s, Fi, mx, lmax, numax, rnumax, T);
                 };
                 const float nu_src = (hm == 2 && src_live) ? nu_s : INFINITY;
                 // one test per lane and 32 columns covers both directions: a pair can be a
@@ -1113,7 +1110,7 @@ __global__ void __launch_bounds__(tc::NUM_THREADS, 1)
                 const int fp = first_pass ? 1 : 0;
                 if (use_l0 && !(th_ok & (1 << fp))) {
                     const float th = screen_theta<N>(k, live, nu_s, rnu_s, Fi, mx, it_lmax, fp ? it_numax1 : it_numax,
-                                                     fp ? it_rnumax1 : it_rnumax, T, e2);
+                                                     fp ? it_rnumax1 : it_rnumax, T);
                     const float thm = (th == -INFINITY) ? th : th + 1e-6f * (fabsf(th) + nu_s + 1.f);
                     if (fp) th_hi1 = thm; else th_hi0 = thm;
                     th_ok |= 1 << fp;

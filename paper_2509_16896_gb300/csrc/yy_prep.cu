@@ -25,7 +25,6 @@
 #include "yy_prep_dims.cuh"
 
 #include <cuda_fp8.h>
-#include <cuda_fp16.h>
 
 #include <type_traits>
 
@@ -105,7 +104,6 @@ __device__ __forceinline__ void prep_rows(const Consts<T>& k, const Bufs<T>& b, 
         mn = first ? (uint8_t)0 : b.mask[i];   // with the row rather than after its reductions
     };
     constexpr bool ahead = NQ <= kShortQ;
-    float emax = 0.f;
     if (ahead) load_row(warp);
     for (long long i = warp; i < k.n_pad; i += nwarps) {
         T* fi = b.f + (size_t)i * rp;
@@ -134,7 +132,6 @@ __device__ __forceinline__ void prep_rows(const Consts<T>& k, const Bufs<T>& b, 
         T div = T(0), nf = T(0), nu = T(0), lw = T(0);
         T hl = T(0);   // noise coefficients: 1/2 log det_+ a(x) = sum of log U_d over U_d > 0
         int on_face = 0;
-        float hq = 0.f, eq = 0.f;   // tensor-core screen: |copy|^2 and |u - copy|^2
         bool done = false;
         if constexpr (std::is_same<T, float>::value && narrow && !first) {
             // the common restart and re-preparation case: cubic drift by the polynomials,
@@ -239,26 +236,12 @@ __device__ __forceinline__ void prep_rows(const Consts<T>& k, const Bufs<T>& b, 
                 if (d >= k.r && b.minv) b.minv[(size_t)i * rp + d] = T(0);
             }
             if (first && b.ubf) {   // (coordinates beyond r are zero)
-                // the screen's copy, and what the copy holds: its norms are the screen's norms,
-                // its distance from u the screen's error radius
                 const float2 v = uu[q];
-                float2 h;
-                if (k.tc_fp8) {   // e4m3 copy of s u, rows of tc_r8 bytes (tail bytes stay zero)
-                    const __nv_fp8x2_storage_t c8 =
+                if (k.tc_fp8)   // e4m3 copy of s u, rows of tc_r8 bytes (tail bytes stay zero)
+                    *reinterpret_cast<__nv_fp8x2_storage_t*>(reinterpret_cast<uint8_t*>(b.ubf) + (size_t)i * k.tc_r8 + dq) =
                         __nv_cvt_float2_to_fp8x2(make_float2(k.tc_s * v.x, k.tc_s * v.y), __NV_SATFINITE, __NV_E4M3);
-                    *reinterpret_cast<__nv_fp8x2_storage_t*>(reinterpret_cast<uint8_t*>(b.ubf) + (size_t)i * k.tc_r8 + dq) = c8;
-                    const float2 d2 = __half22float2(__half2(__nv_cvt_fp8x2_to_halfraw2(c8, __NV_E4M3)));
-                    const float inv = 1.0f / k.tc_s;   // a power of two
-                    h = make_float2(d2.x * inv, d2.y * inv);
-                } else {
-                    const __nv_bfloat162 c16 = __floats2bfloat162_rn(v.x, v.y);
-                    *reinterpret_cast<__nv_bfloat162*>(b.ubf + (size_t)i * rp + dq) = c16;
-                    h = __bfloat1622float2(c16);
-                }
-                cq = fmaf(h.x, h.x, h.y * h.y);
-                hq += cq;
-                const float ex = v.x - h.x, ey = v.y - h.y;
-                eq = fmaf(ex, ex, fmaf(ey, ey, eq));
+                else
+                    *reinterpret_cast<__nv_bfloat162*>(b.ubf + (size_t)i * rp + dq) = __floats2bfloat162_rn(v.x, v.y);
             }
             if (first && b.nu_chunk) {
                 cq = warp_sum(cq);
@@ -274,10 +257,6 @@ __device__ __forceinline__ void prep_rows(const Consts<T>& k, const Bufs<T>& b, 
         }
         if (first) {
             nu = warp_sum(nu);
-            if (b.ubf) {
-                nu = (T)warp_sum(hq);
-                emax = fmaxf(emax, sqrtf(warp_sum(eq)) * 1.00002f);
-            }
             on_face = __any_sync(0xffffffffu, on_face);
         }
         if (lane == 0) {
@@ -304,8 +283,6 @@ __device__ __forceinline__ void prep_rows(const Consts<T>& k, const Bufs<T>& b, 
             }
         }
     }
-    // (a node set re-mapped to wider boxes can only raise it: an upper bound stays one)
-    if (first && b.ubf && lane == 0) atomicMax(reinterpret_cast<int*>(&b.stats->tc_emax), __float_as_int(emax));
 }
 
 // lse_out: also write the block's (max, sum) log-sum-exp partial of the new log-weights to
