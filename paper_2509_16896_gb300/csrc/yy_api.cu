@@ -190,11 +190,12 @@ size_t carve(const yy_config* c, char* base, Bufs<T>* out) {
         b.op = cv.take<float>((size_t)c->n_scales * (size_t)n_pad * (size_t)n_pad * sizeof(float));
         b.op_lsrc = cv.take<float>((size_t)n_pad * sizeof(float));
     }
-    b.dimc = cv.take<T>(8 * (size_t)r_pad * sizeof(T));
+    b.dimc = cv.take<T>(5 * (size_t)r_pad * sizeof(T));
     b.next_centre = cv.take<double>(r_pad * sizeof(double));
     b.next_half = cv.take<double>(r_pad * sizeof(double));
     b.dy_last = cv.take<double>(r_pad * sizeof(double));
     b.part = cv.take<double>(part_bytes(r_pad));
+    b.part_list = cv.take<int>((size_t)kNumPartBlocks * sizeof(int));
     b.stats = cv.take<DevStats>(sizeof(DevStats));
     if (c->precision == YY_PREC_BF16 || c->precision == YY_PREC_FP32_SCREEN)
         b.nu_chunk = cv.take<float>((size_t)n_pad * (r_pad / kColAlign) * sizeof(float));
@@ -558,8 +559,9 @@ yy_status yy_predict(yy_filter* f) {
         if (e == cudaSuccess) e = launch_ksum_scr32(f->kf, f->bf, k1, f->stream, &l);
         f->launches += l;
     } else {
+        e = cudaMemsetAsync(&f->bf.stats->clamps, 0, sizeof(unsigned), f->stream);
         int l = 0;
-        e = launch_ksum_tc(f->kf, f->bf, f->stream, &l);   // (zeroes the counters itself)
+        if (e == cudaSuccess) e = launch_ksum_tc(f->kf, f->bf, f->stream, &l);
         f->launches += l;
         if (e == cudaErrorNotSupported) return YY_ERR_UNSUPPORTED;
     }
@@ -568,22 +570,19 @@ yy_status yy_predict(yy_filter* f) {
     return YY_OK;
 }
 
-// hist_row (device, 2r + 4 doubles, or NULL) receives the step's row of the estimate history.
-static yy_status update_with_row(yy_filter* f, const double* d_dy, double* hist_row) {
+yy_status yy_update(yy_filter* f, const double* d_dy) {
     if (!f || !d_dy) return YY_ERR_ARG;
     if (!f->nodes_ready || !f->predicted) return YY_ERR_STATE;
     if (f->shard_count > 1) return YY_ERR_STATE;   // a shard updates with yy_update_shard
     int l = 0;
     cudaError_t e = f->fp64
-        ? launch_update<double>(f->kd, f->bd, d_dy, f->cfg.restart_interval, f->cfg.ess_frac, hist_row, f->stream, &l)
-        : launch_update<float>(f->kf, f->bf, d_dy, f->cfg.restart_interval, f->cfg.ess_frac, hist_row, f->stream, &l);
+        ? launch_update<double>(f->kd, f->bd, d_dy, f->cfg.restart_interval, f->cfg.ess_frac, f->stream, &l)
+        : launch_update<float>(f->kf, f->bf, d_dy, f->cfg.restart_interval, f->cfg.ess_frac, f->stream, &l);
     f->launches += l;
     if (e != cudaSuccess) return YY_ERR_CUDA;
     f->predicted = false;
     return YY_OK;
 }
-
-yy_status yy_update(yy_filter* f, const double* d_dy) { return update_with_row(f, d_dy, nullptr); }
 
 static yy_status status_from_word(unsigned w) {
     if (w & kStatusTimeout) return YY_ERR_TIMEOUT;
@@ -645,8 +644,14 @@ yy_status yy_run_steps(yy_filter* f, const double* d_dy_all, int64_t K, double* 
     for (int64_t k = 0; k < K; ++k) {
         yy_status st = yy_predict(f);
         if (st != YY_OK) return st;
-        double* row = d_hist ? d_hist + (size_t)k * (2 * r + 4) : nullptr;
-        if ((st = update_with_row(f, d_dy_all + (size_t)k * f->cfg.m, row)) != YY_OK) return st;
+        if ((st = yy_update(f, d_dy_all + (size_t)k * f->cfg.m)) != YY_OK) return st;
+        if (d_hist) {
+            double* row = d_hist + (size_t)k * (2 * r + 4);
+            cudaError_t e = f->fp64 ? launch_record<double>(f->kd, f->bd, row, f->stream)
+                                    : launch_record<float>(f->kf, f->bf, row, f->stream);
+            if (e != cudaSuccess) return YY_ERR_CUDA;
+            f->launches += 1;
+        }
         if ((st = yy_restart(f, YY_RESTART_AUTO, nullptr)) != YY_OK) return st;
     }
     return YY_OK;

@@ -214,7 +214,9 @@ yy_status batch_steps(yy_batch* bt, const double* d_dy_all, int64_t K, double* d
         if (st != YY_OK) return st;
         int l = 0;
         cudaError_t e = launch_update_batch<float>(bt->d_traj, bt->B, bt->r_max, d_dy_all + (size_t)k * bt->M,
-                                                   d_hist ? d_hist + (size_t)k * bt->H : nullptr, bt->nbu, bt->stream, &l);
+                                                   bt->nbu, bt->stream, &l);
+        if (e == cudaSuccess && d_hist)
+            e = launch_record_batch<float>(bt->d_traj, bt->B, d_hist + (size_t)k * bt->H, bt->stream, &l);
         if (e == cudaSuccess)
             e = launch_restart_batch<float>(bt->d_traj, bt->B, bt->r_max, bt->n_pad_max, bt->nbu, bt->stream, &l);
         bt->launches += l;

@@ -41,7 +41,7 @@ struct DevStats {
     int last_restarted;  // 1 if the last yy_restart call re-centred the box
     int scale_changed;   // 1 while a restart re-maps the nodes to new half-widths
     double c_ref;        // offset of the predicted log-weights (moves with the box volume)
-    int norm_flag;       // 1 while the weights of a restart wait for their normalisation
+    int part_count;      // entries of part_list
     // tensor-core screen: stages (64 BF16 or 128 e4m3 coordinates) of the first pass and its controller
     int tc_nk1;          // 0 = not chosen yet
     int tc_streak;       // consecutive clean predictions at the current length
@@ -116,13 +116,13 @@ struct Bufs {
     float* op_lsrc;       // [n_pad] source terms of the materialised apply (log2 e ell_s, -inf if not live)
     T* minv;              // [n_pad][r_pad] noise coefficients: a(x)^+ (diagonal) at every node
     T* hld;               // [n_pad] noise coefficients: 1/2 log det_+ a(x)
-    T* dimc;              // [8][r_pad] per-dimension constants of the preparation pass:
-                          // centre head, tail, Gaussian restart 1 / (2 var), cos c, sin c, the
-                          // boundary as a float, centre minus prior mean (head, tail)
+    T* dimc;              // [5][r_pad] per-dimension constants of the preparation pass:
+                          // centre head, tail, Gaussian restart 1 / (2 var), cos c, sin c
     double* next_centre;  // [r_pad] box of the restart in progress
     double* next_half;    // [r_pad]
     double* dy_last;      // [r_pad] observation increment of the last update
     double* part;         // reduction partials
+    int* part_list;       // [kNumPartBlocks] moment partials with weight, in block order
     DevStats* stats;
     // tensor-core screen scratch (BF16 precision only)
     float* nu_chunk;      // [n_pad][r_pad / 64] |u_i|^2 per chunk of 64 coordinates (BF16 only)
@@ -213,8 +213,11 @@ int tc_pair_max_clusters();
 int tc_max_split();
 
 template <typename T>
+cudaError_t launch_record(const Consts<T>& k, const Bufs<T>& b, double* hist_row, cudaStream_t s);
+
+template <typename T>
 cudaError_t launch_update(const Consts<T>& k, const Bufs<T>& b, const double* dy,
-                          int restart_interval, double ess_frac, double* hist_row, cudaStream_t s, int* launches);
+                          int restart_interval, double ess_frac, cudaStream_t s, int* launches);
 
 template <typename T>
 cudaError_t launch_restart(const Consts<T>& k, const Bufs<T>& b, int mode, int init_kind, double base_R,
@@ -237,11 +240,13 @@ const float* mlp_output(const struct ::yy_mlp* net);
 
 // Batched launches: one launch covers every trajectory (grid.y = trajectory).
 template <typename T>
-cudaError_t launch_update_batch(const Traj<T>* d_traj, int B, int r_max, const double* dy_row, double* hist_row,
+cudaError_t launch_update_batch(const Traj<T>* d_traj, int B, int r_max, const double* dy_row,
                                 int nbu, cudaStream_t s, int* launches);
 template <typename T>
 cudaError_t launch_restart_batch(const Traj<T>* d_traj, int B, int r_max, long long n_pad_max,
                                  int nbu, cudaStream_t s, int* launches);
+template <typename T>
+cudaError_t launch_record_batch(const Traj<T>* d_traj, int B, double* hist_row, cudaStream_t s, int* launches);
 template <typename T>
 cudaError_t launch_reset_batch(const Traj<T>* d_traj, int B, cudaStream_t s, int* launches);
 bool make_tc_map(void* map /* CUtensorMap */, const void* base, long long rows, int cols, int box_rows, bool fp8);

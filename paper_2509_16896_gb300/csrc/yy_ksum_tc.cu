@@ -325,14 +325,7 @@ __device__ __forceinline__ void colprep_body(const Consts<float>& k, const Bufs<
     }
 }
 
-// Also zeroes the prediction's counters.
-__global__ void __launch_bounds__(128) k_tc_colprep(Consts<float> k, Bufs<float> b) {
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        b.stats->clamps = 0u;
-        b.stats->candidates = 0ull;
-    }
-    colprep_body(k, b, blockIdx.x);
-}
+__global__ void __launch_bounds__(128) k_tc_colprep(Consts<float> k, Bufs<float> b) { colprep_body(k, b, blockIdx.x); }
 
 __global__ void __launch_bounds__(128) kb_tc_colprep(const Traj<float>* __restrict__ tr) {
     const Traj<float>& t = tr[blockIdx.y];
@@ -1293,32 +1286,26 @@ __device__ __forceinline__ void tc_merge_body(const Consts<float>& k, const Bufs
         if (b.mask[i]) { b.logw_pred[i] = -INFINITY; continue; }
         const int ns = k.tc_sym ? tc_sym_splits(nst - (int)(i / 256), k.tc_split_len) : nsplit;
         float mx[N], sm[N];
-        auto add = [&](int j, float m2, float s2) {
-            if (m2 == -INFINITY || !(s2 > 0.f)) return;
-            if (mx[j] == -INFINITY) { mx[j] = m2; sm[j] = s2; }
-            else if (m2 > mx[j]) { sm[j] = sm[j] * expf(mx[j] - m2) + s2; mx[j] = m2; }
-            else sm[j] += s2 * expf(m2 - mx[j]);
-        };
 #pragma unroll
-        for (int j = 0; j < N; ++j) { mx[j] = -INFINITY; sm[j] = 0.f; }
-        unsigned long long xw[N];
-#pragma unroll
-        for (int j = 0; j < N; ++j) xw[j] = k.tc_sym ? b.tc_xlse[(size_t)i * kMaxScales + j] : 0ull;
-        for (int q0 = 0; q0 < ns; q0 += 4) {   // four ranges' states loaded before any is used
-            float2 v[4][N];
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-#pragma unroll
-                for (int j = 0; j < N; ++j)
-                    v[q][j] = (q0 + q < ns) ? *reinterpret_cast<const float2*>(part_slot(b, i, q0 + q, j))
-                                            : make_float2(-INFINITY, 0.f);
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-#pragma unroll
-                for (int j = 0; j < N; ++j) add(j, v[q][j].x, v[q][j].y);
+        for (int j = 0; j < N; ++j) {
+            float m = -INFINITY, s = 0.f;
+            auto add = [&](float m2, float s2) {
+                if (m2 == -INFINITY || !(s2 > 0.f)) return;
+                if (m == -INFINITY) { m = m2; s = s2; }
+                else if (m2 > m) { s = s * expf(m - m2) + s2; m = m2; }
+                else s += s2 * expf(m2 - m);
+            };
+            for (int q = 0; q < ns; ++q) {
+                const float* ps = part_slot(b, i, q, j);
+                add(ps[0], ps[1]);
+            }
+            if (k.tc_sym) {
+                const unsigned long long w = b.tc_xlse[(size_t)i * kMaxScales + j];
+                add(__uint_as_float((uint32_t)w), __uint_as_float((uint32_t)(w >> 32)));
+            }
+            mx[j] = m;
+            sm[j] = s;
         }
-#pragma unroll
-        for (int j = 0; j < N; ++j) add(j, __uint_as_float((uint32_t)xw[j]), __uint_as_float((uint32_t)(xw[j] >> 32)));
         b.logw_pred[i] = combine_scales<float, N>(k, mx, sm, b.divf[i], b.logw[i], b.stats->c_ref, &b.stats->clamps);
     }
 }
@@ -1481,9 +1468,10 @@ cudaError_t launch_ksum_tc(const Consts<float>& k, const Bufs<float>& b, cudaStr
     const int cols = k.tc_fp8 ? k.tc_r8 : k.r_pad;
     if (!make_tc_map(&ma, b.ubf, k.n_pad, cols, tc::BM, k.tc_fp8) || !make_tc_map(&mb, b.ubf, k.n_pad, cols, 256, k.tc_fp8))
         return cudaErrorNotSupported;
-    k_tc_colprep<<<(unsigned)(k.n_pad / 128), 128, 0, s>>>(k, b);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = cudaMemsetAsync(&b.stats->candidates, 0, sizeof(unsigned long long), s);
     if (e != cudaSuccess) return e;
+    k_tc_colprep<<<(unsigned)(k.n_pad / 128), 128, 0, s>>>(k, b);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (k.tc_sym) {
         k_tc_colprep2<<<(unsigned)(k.n_pad / 128), 128, 0, s>>>(k, b);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
@@ -1495,13 +1483,12 @@ cudaError_t launch_ksum_tc(const Consts<float>& k, const Bufs<float>& b, cudaStr
     if (e != cudaSuccess) return e;
     int l = k.tc_sym ? 3 : 2;
     if (b.tc_splits > 1 || k.tc_sym) {
-        // a row per thread in small blocks, so that every SM gets some
-        const unsigned g = (unsigned)std::min<long long>((k.n + 63) / 64, 4096);
+        const unsigned g = (unsigned)std::min<long long>((k.n + 255) / 256, 1024);
         switch (k.N) {
-            case 1: k_tc_merge<1><<<g, 64, 0, s>>>(k, b, b.tc_splits); break;
-            case 2: k_tc_merge<2><<<g, 64, 0, s>>>(k, b, b.tc_splits); break;
-            case 3: k_tc_merge<3><<<g, 64, 0, s>>>(k, b, b.tc_splits); break;
-            case 4: k_tc_merge<4><<<g, 64, 0, s>>>(k, b, b.tc_splits); break;
+            case 1: k_tc_merge<1><<<g, 256, 0, s>>>(k, b, b.tc_splits); break;
+            case 2: k_tc_merge<2><<<g, 256, 0, s>>>(k, b, b.tc_splits); break;
+            case 3: k_tc_merge<3><<<g, 256, 0, s>>>(k, b, b.tc_splits); break;
+            case 4: k_tc_merge<4><<<g, 256, 0, s>>>(k, b, b.tc_splits); break;
         }
         l += 1;
     }

@@ -21,7 +21,6 @@
 // comes from the angle-addition form of yy_drift.cuh; in float64 from sincos.
 #include "yy_internal.cuh"
 #include "yy_drift.cuh"
-#include "yy_lse.cuh"
 #include "yy_prep_dims.cuh"
 
 #include <cuda_fp8.h>
@@ -38,7 +37,6 @@ __device__ __forceinline__ T warp_sum(T v) {
 }
 
 constexpr int kRowQ = YY_MAX_DIM / 64;   // float2 per lane of the longest row
-constexpr int kShortQ = 2;               // and of short rows (r <= 128)
 
 // Drift component d of the large-scale test's model at x_d with neighbour x_{d+1} (nb = 0
 // for the last coordinate: the bidiagonal matrices have no entry there), and the
@@ -76,36 +74,22 @@ __device__ __forceinline__ double exp_w<double>(double x) { return exp(x); }
 
 // The pass proper, compiled per mode and per "first" (node-only quantities too), so that
 // the restart pass carries none of the other modes' float64 arithmetic.
-// NQ: float2 per lane of the longest row the instance takes.  Short rows (NQ = 2) are bound by
-// latency, so a warp's next row is loaded under the arithmetic of this one.
-template <typename T, int mode, bool first, bool narrow, int NQ>
+template <typename T, int mode, bool first, bool narrow>
 __device__ __forceinline__ void prep_rows(const Consts<T>& k, const Bufs<T>& b, double prior_mean,
                                           double prior_var, int bid, int nblk, const T* s_hi, const T* s_lo,
-                                          const T* s_iv, const T* s_cc, const T* s_sc, const float* s_face,
-                                          const float* s_zh, const float* s_zl, T& lse_m, T& lse_s) {
+                                          const T* s_iv, const T* s_cc, const T* s_sc, T& lse_m,
+                                          T& lse_s) {
     const int rp = k.r_pad;
     const int lane = threadIdx.x & 31;
     const long long warp = (bid * (long long)blockDim.x + threadIdx.x) >> 5;
     const long long nwarps = ((long long)nblk * blockDim.x) >> 5;
-    const double* cen = b.centre;   // (float64 prior)
-    // prior, float32: 1 / (2 var) as two floats
-    const double iv2 = (mode == kPrepInit) ? 0.5 / prior_var : 0.0;
-    const float ivh = (float)iv2, ivl = (float)(iv2 - (double)ivh);
+    const double* cen = (mode == kPrepRestart) ? b.next_centre : b.centre;
+    const double* halfw = (mode == kPrepRestart) ? b.next_half : b.halfwidth;
     const int nq = rp >> 6;   // float2 per lane
     const bool cubic = k.model == YY_MODEL_CUBIC;
     const bool e1 = k.model == YY_MODEL_PAPER_E1;
-    float2 un[NQ];
-    uint8_t mn = 0;
-    auto load_row = [&](long long i) {
-        if (i >= k.n) return;
-        const float2* ui2 = reinterpret_cast<const float2*>(b.u + (size_t)i * rp);
-#pragma unroll
-        for (int q = 0; q < NQ; ++q) un[q] = (q < nq) ? ui2[lane + 32 * q] : make_float2(0.f, 0.f);
-        mn = first ? (uint8_t)0 : b.mask[i];   // with the row rather than after its reductions
-    };
-    constexpr bool ahead = NQ <= kShortQ;
-    if (ahead) load_row(warp);
     for (long long i = warp; i < k.n_pad; i += nwarps) {
+        const float* ui = b.u + (size_t)i * rp;
         T* fi = b.f + (size_t)i * rp;
         if (i >= k.n) {  // padding rows: inert
             if (b.store_f)
@@ -123,12 +107,13 @@ __device__ __forceinline__ void prep_rows(const Consts<T>& k, const Bufs<T>& b, 
                 for (int c = lane; c < nq; c += 32) b.nu_chunk[(size_t)i * nq + c] = 0.f;
             continue;
         }
-        if (!ahead) load_row(i);   // the whole row first
-        float2 uu[NQ];
+        // the whole row first: up to kRowQ loads in flight per lane
+        const float2* ui2 = reinterpret_cast<const float2*>(ui);
+        float2 uu[kRowQ];
 #pragma unroll
-        for (int q = 0; q < NQ; ++q) uu[q] = un[q];
-        const uint8_t mk = mn;
-        if (ahead) load_row(i + nwarps);
+        for (int q = 0; q < kRowQ; ++q) uu[q] = (q < nq) ? ui2[lane + 32 * q] : make_float2(0.f, 0.f);
+        // the stored boundary mask, loaded with the row rather than after its reductions
+        const uint8_t mk = first ? (uint8_t)0 : b.mask[i];
         T div = T(0), nf = T(0), nu = T(0), lw = T(0);
         T hl = T(0);   // noise coefficients: 1/2 log det_+ a(x) = sum of log U_d over U_d > 0
         int on_face = 0;
@@ -139,7 +124,7 @@ __device__ __forceinline__ void prep_rows(const Consts<T>& k, const Bufs<T>& b, 
             // term), so no per-element tests; per-dimension constants as float2 pairs
             if (cubic && k.noise == YY_NOISE_UNIT) {
 #pragma unroll
-                for (int q = 0; q < NQ; ++q) {
+                for (int q = 0; q < kRowQ; ++q) {
                     if (q >= nq) break;   // uniform over the warp
                     const int d = 64 * q + 2 * lane;
                     const float2 cc = *reinterpret_cast<const float2*>(s_cc + d);
@@ -159,7 +144,7 @@ __device__ __forceinline__ void prep_rows(const Consts<T>& k, const Bufs<T>& b, 
             }
         }
 #pragma unroll
-        for (int q = 0; q < NQ; ++q) {
+        for (int q = 0; q < kRowQ; ++q) {
             if (done) break;
             if (q >= nq) break;   // uniform over the warp
             const int dq = 64 * q + 2 * lane;
@@ -169,7 +154,7 @@ __device__ __forceinline__ void prep_rows(const Consts<T>& k, const Bufs<T>& b, 
             float u_next = 0.f;
             if (e1) {
                 const float from_lane = __shfl_down_sync(0xffffffffu, uu[q].x, 1);
-                const float from_next = __shfl_sync(0xffffffffu, (q + 1 < NQ) ? uu[q + 1 < NQ ? q + 1 : q].x : 0.f, 0);
+                const float from_next = __shfl_sync(0xffffffffu, (q + 1 < kRowQ) ? uu[q + 1 < kRowQ ? q + 1 : q].x : 0.f, 0);
                 u_next = (lane < 31) ? from_lane : ((q + 1 < nq) ? from_next : 0.f);
             }
 #pragma unroll
@@ -215,33 +200,23 @@ __device__ __forceinline__ void prep_rows(const Consts<T>& k, const Bufs<T>& b, 
                     if constexpr (first) {
                         nu += (T)uf * (T)uf;
                         cq = fmaf(uf, uf, cq);
-                        if (fabsf(uf) >= s_face[d]) on_face = 1;
+                        const double R = halfw[d];
+                        if (fabs((double)uf) >= R - 1e-12 * R) on_face = 1;
                     }
-                    if constexpr (mode == kPrepInit && std::is_same<T, float>::value) {
-                        // z^2 / (2 var), z = c + u - mu0, rounded once to float: z, its square and
-                        // the quotient as pairs of floats (relative error below 2^-44), since six
-                        // float64 operations per coordinate are what this pass would wait for
-                        // (r = 1000, n = 65536: 2.0 ms, 0.38 so)
-                        const float a = s_zh[d], zs = a + uf, bb = zs - a;
-                        const float zt = ((a - (zs - bb)) + (uf - bb)) + s_zl[d];
-                        const float p = zs * zs, pl = fmaf(2.f * zs, zt, fmaf(zs, zs, -p));
-                        const float t = p * ivh;
-                        lw -= t + (fmaf(p, ivh, -t) + fmaf(pl, ivh, p * ivl));
-                    } else if constexpr (mode == kPrepInit) {
+                    if constexpr (mode == kPrepInit) {
                         const double z = cen[d] + (double)uf - prior_mean;
                         lw -= (T)(0.5 * z * z / prior_var);
                     }
                 }
+                if (first && b.ubf) {
+                    if (k.tc_fp8)   // e4m3 copy of s u, rows of tc_r8 bytes (tail bytes stay zero)
+                        reinterpret_cast<uint8_t*>(b.ubf)[(size_t)i * k.tc_r8 + d] = (uint8_t)__nv_cvt_float_to_fp8(
+                            d < k.r ? k.tc_s * uf : 0.0f, __NV_SATFINITE, __NV_E4M3);
+                    else
+                        b.ubf[(size_t)i * rp + d] = __float2bfloat16_rn(d < k.r ? uf : 0.0f);
+                }
                 if (b.store_f) fi[d] = fv;
                 if (d >= k.r && b.minv) b.minv[(size_t)i * rp + d] = T(0);
-            }
-            if (first && b.ubf) {   // (coordinates beyond r are zero)
-                const float2 v = uu[q];
-                if (k.tc_fp8)   // e4m3 copy of s u, rows of tc_r8 bytes (tail bytes stay zero)
-                    *reinterpret_cast<__nv_fp8x2_storage_t*>(reinterpret_cast<uint8_t*>(b.ubf) + (size_t)i * k.tc_r8 + dq) =
-                        __nv_cvt_float2_to_fp8x2(make_float2(k.tc_s * v.x, k.tc_s * v.y), __NV_SATFINITE, __NV_E4M3);
-                else
-                    *reinterpret_cast<__nv_bfloat162*>(b.ubf + (size_t)i * rp + dq) = __floats2bfloat162_rn(v.x, v.y);
             }
             if (first && b.nu_chunk) {
                 cq = warp_sum(cq);
@@ -287,17 +262,14 @@ __device__ __forceinline__ void prep_rows(const Consts<T>& k, const Bufs<T>& b, 
 
 // lse_out: also write the block's (max, sum) log-sum-exp partial of the new log-weights to
 // b.part[2 bid], b.part[2 bid + 1] (restart and init passes).
-template <typename T, int NQ>
+template <typename T>
 __device__ __forceinline__ void prep_body(const Consts<T>& k, const Bufs<T>& b, int mode, int first,
                                           double prior_mean, double prior_var, int bid, int nblk, bool lse_out) {
     if (mode == kPrepRestart && b.stats->restart_flag == 0) return;
     // a restart that re-mapped the nodes to new half-widths also redoes the node-only
     // quantities (|u|^2, mask against the new faces, bf16 copy)
     if (mode == kPrepRestart && b.stats->scale_changed) first = 1;
-    constexpr int MD = NQ * 64;
-    __shared__ T s_hi[MD], s_lo[MD], s_iv[MD], s_cc[MD], s_sc[MD];
-    constexpr int MZ = std::is_same<T, float>::value ? MD : 1;   // (float32 prior)
-    __shared__ float s_face[MD], s_zh[MZ], s_zl[MZ];
+    __shared__ T s_hi[YY_MAX_DIM], s_lo[YY_MAX_DIM], s_iv[YY_MAX_DIM], s_cc[YY_MAX_DIM], s_sc[YY_MAX_DIM];
     const int rp = k.r_pad;
     for (int d = threadIdx.x; d < rp; d += blockDim.x) {
         s_hi[d] = b.dimc[d];
@@ -305,13 +277,6 @@ __device__ __forceinline__ void prep_body(const Consts<T>& k, const Bufs<T>& b, 
         s_iv[d] = b.dimc[2 * rp + d];
         s_cc[d] = b.dimc[3 * rp + d];
         s_sc[d] = b.dimc[4 * rp + d];
-        if (first) {
-            s_face[d] = (float)b.dimc[5 * rp + d];
-            if constexpr (MZ > 1) {
-                s_zh[d] = b.dimc[6 * rp + d];
-                s_zl[d] = b.dimc[7 * rp + d];
-            }
-        }
     }
     // every dimension inside the polynomials' range: no per-element fallback test
     int my_narrow = 1;
@@ -319,15 +284,13 @@ __device__ __forceinline__ void prep_body(const Consts<T>& k, const Bufs<T>& b, 
     const int narrow = __syncthreads_and(my_narrow);
     T lse_m = T(-INFINITY), lse_s = T(0);
 #define YY_PREP_ROWS(M, F, W) \
-    prep_rows<T, M, F, W, NQ>(k, b, prior_mean, prior_var, bid, nblk, s_hi, s_lo, s_iv, s_cc, s_sc, s_face, s_zh, s_zl, lse_m, lse_s)
+    prep_rows<T, M, F, W>(k, b, prior_mean, prior_var, bid, nblk, s_hi, s_lo, s_iv, s_cc, s_sc, lse_m, lse_s)
     if (mode == kPrepRestart) {
         if (first) YY_PREP_ROWS(kPrepRestart, true, false);
         else if (narrow) YY_PREP_ROWS(kPrepRestart, false, true);
         else YY_PREP_ROWS(kPrepRestart, false, false);
     } else if (mode == kPrepInit) {
-        if (first && narrow) YY_PREP_ROWS(kPrepInit, true, true);
-        else if (first) YY_PREP_ROWS(kPrepInit, true, false);
-        else YY_PREP_ROWS(kPrepInit, false, false);
+        if (first) YY_PREP_ROWS(kPrepInit, true, false); else YY_PREP_ROWS(kPrepInit, false, false);
     } else {
         if (first) YY_PREP_ROWS(kPrepOnly, true, false);
         else if (narrow) YY_PREP_ROWS(kPrepOnly, false, true);
@@ -339,23 +302,29 @@ __device__ __forceinline__ void prep_body(const Consts<T>& k, const Bufs<T>& b, 
         const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
         if (lane == 0) { sm_m[wib] = (double)lse_m; sm_s[wib] = (double)lse_s; }
         __syncthreads();
-        if (threadIdx.x < 32) {
-            double M, S;
-            lse_merge8(sm_m[lane & 7], sm_s[lane & 7], M, S);
-            if (lane == 0) { b.part[2 * bid] = M; b.part[2 * bid + 1] = S; }
+        if (threadIdx.x == 0) {
+            double M = -INFINITY, S = 0.0;
+            for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
+                const double m2 = sm_m[w], s2 = sm_s[w];
+                if (m2 == -INFINITY) continue;
+                if (M == -INFINITY) { M = m2; S = s2; }
+                else if (m2 > M) { S = S * exp(M - m2) + s2; M = m2; }
+                else S += s2 * exp(m2 - M);
+            }
+            b.part[2 * bid] = M;
+            b.part[2 * bid + 1] = S;
         }
     }
 }
 
 template <typename T>
-__global__ void k_prep_dims(Consts<T> k, Bufs<T> b, int mode, int init_kind, double prior_mean) {
-    prep_dims_body<T>(k, b, mode, init_kind, blockIdx.x, gridDim.x, prior_mean);
+__global__ void k_prep_dims(Consts<T> k, Bufs<T> b, int mode, int init_kind) {
+    prep_dims_body<T>(k, b, mode, init_kind, blockIdx.x, gridDim.x);
 }
-template <typename T, int NQ>
-__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 1) k_prep(const __grid_constant__ Consts<T> k,
-                                                                      const __grid_constant__ Bufs<T> b, int mode,
-                                                                      int first, double prior_mean, double prior_var) {
-    prep_body<T, NQ>(k, b, mode, first, prior_mean, prior_var, blockIdx.x, gridDim.x, true);
+template <typename T>
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 1) k_prep(Consts<T> k, Bufs<T> b, int mode, int first, double prior_mean,
+                                              double prior_var) {
+    prep_body<T>(k, b, mode, first, prior_mean, prior_var, blockIdx.x, gridDim.x, true);
 }
 // batched restart preparation: trajectory = blockIdx.y
 template <typename T>
@@ -363,23 +332,22 @@ __global__ void kb_prep_dims(const Traj<T>* __restrict__ tr) {
     const Traj<T>& t = tr[blockIdx.y];
     prep_dims_body<T>(t.k, t.b, kPrepRestart, t.restart_init, 0, 1);
 }
-template <typename T, int NQ>
+template <typename T>
 __global__ void __launch_bounds__(256) kb_prep(const Traj<T>* __restrict__ tr) {
     const Traj<T>& t = tr[blockIdx.y];
-    prep_body<T, NQ>(t.k, t.b, kPrepRestart, 0, 0.0, 1.0, blockIdx.x, gridDim.x, false);
+    prep_body<T>(t.k, t.b, kPrepRestart, 0, 0.0, 1.0, blockIdx.x, gridDim.x, false);
 }
 
 template <typename T>
-cudaError_t launch_prep_restart_batch(const Traj<T>* d_traj, int B, int r_max, long long n_pad_max, cudaStream_t s) {
+cudaError_t launch_prep_restart_batch(const Traj<T>* d_traj, int B, long long n_pad_max, cudaStream_t s) {
     kb_prep_dims<T><<<dim3(1, B), 256, 0, s>>>(d_traj);
     long long blocks = (n_pad_max * 32 + 255) / 256;
     if (blocks > 64) blocks = 64;
-    if (r_max <= 64 * kShortQ) kb_prep<T, kShortQ><<<dim3((unsigned)blocks, B), 256, 0, s>>>(d_traj);
-    else kb_prep<T, kRowQ><<<dim3((unsigned)blocks, B), 256, 0, s>>>(d_traj);
+    kb_prep<T><<<dim3((unsigned)blocks, B), 256, 0, s>>>(d_traj);
     return cudaGetLastError();
 }
-template cudaError_t launch_prep_restart_batch<float>(const Traj<float>*, int, int, long long, cudaStream_t);
-template cudaError_t launch_prep_restart_batch<double>(const Traj<double>*, int, int, long long, cudaStream_t);
+template cudaError_t launch_prep_restart_batch<float>(const Traj<float>*, int, long long, cudaStream_t);
+template cudaError_t launch_prep_restart_batch<double>(const Traj<double>*, int, long long, cudaStream_t);
 
 // Blocks of the single-filter preparation pass (one warp per row, at most 8 per SM); also
 // the number of log-sum-exp partials it writes.
@@ -392,26 +360,18 @@ int prep_grid(long long n_pad) {
 }
 
 template <typename T>
-void launch_rows(const Consts<T>& k, const Bufs<T>& b, int mode, int first, double prior_mean, double prior_var,
-                 cudaStream_t s) {
-    const unsigned g = (unsigned)prep_grid(k.n_pad);
-    if (k.r_pad <= 64 * kShortQ) k_prep<T, kShortQ><<<g, 256, 0, s>>>(k, b, mode, first, prior_mean, prior_var);
-    else k_prep<T, kRowQ><<<g, 256, 0, s>>>(k, b, mode, first, prior_mean, prior_var);
-}
-
-template <typename T>
 cudaError_t launch_prep_mode(const Consts<T>& k, const Bufs<T>& b, int mode, bool first,
                              double prior_mean, double prior_var, int init_kind, cudaStream_t s) {
     // float64 cosine and sine per dimension: one 32-thread block per 32 dimensions
-    k_prep_dims<T><<<(unsigned)((k.r_pad + 31) / 32), 32, 0, s>>>(k, b, mode, init_kind, prior_mean);
-    launch_rows<T>(k, b, mode, first ? 1 : 0, prior_mean, prior_var, s);
+    k_prep_dims<T><<<(unsigned)((k.r_pad + 31) / 32), 32, 0, s>>>(k, b, mode, init_kind);
+    k_prep<T><<<(unsigned)prep_grid(k.n_pad), 256, 0, s>>>(k, b, mode, first ? 1 : 0, prior_mean, prior_var);
     return cudaGetLastError();
 }
 
 // The rows only (the per-dimension constants already written, as by the restart head).
 template <typename T>
 cudaError_t launch_prep_rows(const Consts<T>& k, const Bufs<T>& b, int mode, cudaStream_t s) {
-    launch_rows<T>(k, b, mode, 0, 0.0, 1.0, s);
+    k_prep<T><<<(unsigned)prep_grid(k.n_pad), 256, 0, s>>>(k, b, mode, 0, 0.0, 1.0);
     return cudaGetLastError();
 }
 template cudaError_t launch_prep_rows<float>(const Consts<float>&, const Bufs<float>&, int, cudaStream_t);

@@ -36,16 +36,13 @@ __device__ __forceinline__ void dim_cos_sin<double>(double c, double* cs, double
 // half-width is too wide for the polynomials of yy_drift.cuh).
 template <typename T>
 __device__ __forceinline__ void prep_dims_body(const Consts<T>& k, const Bufs<T>& b, int mode, int init_kind,
-                                               int bid, int nblk, double prior_mean = 0.0) {
+                                               int bid, int nblk) {
     if (mode == kPrepRestart && b.stats->restart_flag == 0) return;
     const double* cen = (mode == kPrepRestart) ? b.next_centre : b.centre;
     const double* half = (mode == kPrepRestart) ? b.next_half : b.halfwidth;
     const int rp = k.r_pad;
     for (int d = bid * blockDim.x + threadIdx.x; d < rp; d += nblk * blockDim.x) {
         T hi = T(0), lo = T(0), iv = T(0), cc = T(0), sc = T(0);   // padded: u = 0 gives f = 0
-        // node-only passes: the smallest float |u_d| on the boundary (u is a float number, so the
-        // comparison is the float64 one), and the centre relative to the prior's as two floats
-        float face = INFINITY, zh = 0.f, zl = 0.f;
         if (d < k.r) {
             const double c = cen[d];
             hi = (T)c;
@@ -58,19 +55,12 @@ __device__ __forceinline__ void prep_dims_body(const Consts<T>& k, const Bufs<T>
             dim_cos_sin<T>(c, &cs, &sn);
             cc = (half[d] <= kPolyMaxU) ? cs : (T)NAN;
             sc = sn;
-            face = __double2float_ru(half[d] - 1e-12 * half[d]);
-            const double z = c - prior_mean;
-            zh = (float)z;
-            zl = (float)(z - (double)zh);
         }
         b.dimc[d] = hi;
         b.dimc[rp + d] = lo;
         b.dimc[2 * rp + d] = iv;
         b.dimc[3 * rp + d] = cc;
         b.dimc[4 * rp + d] = sc;
-        b.dimc[5 * rp + d] = (T)face;
-        b.dimc[6 * rp + d] = (T)zh;
-        b.dimc[7 * rp + d] = (T)zl;
     }
 }
 
