@@ -117,23 +117,54 @@ __global__ void __launch_bounds__(128) k_gemm_tc(int M, int N, int K, const floa
     const bool b_kcol = (sbk == 1);
     bool ok = true;
     int kc_fail = 0;
-    for (int kc = 0; kc < nchunks; ++kc) {
-        const int k0 = kc * GK;
-        for (int q = 0; q < GM * GK / 128; ++q) {
-            const int e = tid + 128 * q;
-            const int row = a_krow ? (e >> 6) : (e & (GM - 1));
-            const int kk = a_krow ? (e & 63) : (e >> 7);
-            const long long m = m0 + row, k = k0 + kk;
-            const float v = (m < M && k < K) ? A[m * sam + k * sak] : 0.f;
-            *reinterpret_cast<__nv_bfloat16*>(sA + sw128_offset(row, kk)) = __float2bfloat16_rn(v);
-        }
-        for (int q = 0; q < GN * GK / 128; ++q) {
+    // B elements of a chunk: 32 per thread, all loaded before any is used, and the next chunk's
+    // under this one's MMAs
+    constexpr int NB = GN * GK / 128;
+    float bv[NB];
+    auto load_b = [&](int kc) {
+#pragma unroll
+        for (int q = 0; q < NB; ++q) {
             const int e = tid + 128 * q;
             const int col = b_kcol ? (e >> 6) : (e & (GN - 1));
             const int kk = b_kcol ? (e & 63) : (e >> 6);
-            const long long n = n0 + col, k = k0 + kk;
-            const float v = (n < N && k < K) ? Bm[k * sbk + n * sbn] : 0.f;
-            *reinterpret_cast<__nv_bfloat16*>(sB + sw128_offset(col, kk)) = __float2bfloat16_rn(v);
+            const long long n = n0 + col, k = (long long)kc * GK + kk;
+            bv[q] = (n < N && k < K) ? Bm[k * sbk + n * sbn] : 0.f;
+        }
+    };
+    // rows beyond the matrix are zeroed once (a restart's proposal has one row of 128)
+    const int rows = (int)(M - m0 < GM ? M - m0 : GM);
+    if (rows < GM)
+        for (int e = tid; e < GM * GK * 2 / 16; e += 128) reinterpret_cast<uint4*>(sA)[e] = make_uint4(0u, 0u, 0u, 0u);
+    if (nchunks > 0) load_b(0);
+    if (rows < GM) __syncthreads();
+    for (int kc = 0; kc < nchunks; ++kc) {
+        const int k0 = kc * GK;
+        const int na = a_krow ? (rows * GK + 127) / 128 : GM * GK / 128;
+        for (int q0 = 0; q0 < na; q0 += 8) {
+            float av[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const int e = tid + 128 * (q0 + j);
+                const int row = a_krow ? (e >> 6) : (e & (GM - 1));
+                const int kk = a_krow ? (e & 63) : (e >> 7);
+                const long long k = k0 + kk;
+                av[j] = (q0 + j < na && row < rows && k < K) ? A[(m0 + row) * sam + k * sak] : 0.f;
+            }
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const int e = tid + 128 * (q0 + j);
+                const int row = a_krow ? (e >> 6) : (e & (GM - 1));
+                const int kk = a_krow ? (e & 63) : (e >> 7);
+                if (q0 + j < na && row < rows)
+                    *reinterpret_cast<__nv_bfloat16*>(sA + sw128_offset(row, kk)) = __float2bfloat16_rn(av[j]);
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < NB; ++q) {
+            const int e = tid + 128 * q;
+            const int col = b_kcol ? (e >> 6) : (e & (GN - 1));
+            const int kk = b_kcol ? (e & 63) : (e >> 6);
+            *reinterpret_cast<__nv_bfloat16*>(sB + sw128_offset(col, kk)) = __float2bfloat16_rn(bv[q]);
         }
         // generic-proxy writes of shared memory become visible to the tensor cores' reads
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -146,6 +177,7 @@ __global__ void __launch_bounds__(128) k_gemm_tc(int M, int N, int K, const floa
                 mma_bf16(tmem, sw128_desc(a0 + kk * 32), sw128_desc(b0 + kk * 32), kGemmIdesc, (kc | kk) != 0 ? 1u : 0u);
             mma_commit(&bar);
         }
+        if (kc + 1 < nchunks) load_b(kc + 1);
         // every thread waits for the chunk's MMAs before shared memory is written again
         if (!gemm_wait(&bar, (uint32_t)(kc & 1), kGemmWaitNs)) s_fail = 1;
         __syncthreads();
