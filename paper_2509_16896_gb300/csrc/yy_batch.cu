@@ -40,6 +40,8 @@ struct yy_batch {
     int4* d_items;
     int* d_cta_start;
     int max_items, max_grid;
+    int2* d_pair_items;             // float32 form: (member, target block)
+    int n_pair_items;
     // schedule
     int bn, grid, n_items;
     std::vector<int> path;          // per filter: 0 = tcgen05 screen, 1 = FP32 form
@@ -78,12 +80,20 @@ long long total_items(const yy_config* cfgs, int B) {
     return t * 8;                                                    // up to 8 source splits
 }
 
+// Items of the float32 form: target blocks.
+long long total_pair_items(const yy_config* cfgs, int B) {
+    long long t = 0;
+    for (int b = 0; b < B; ++b) t += pair_batch_blocks(cfgs[b].n);
+    return t;
+}
+
 size_t header_bytes(const yy_config* cfgs, int B) {
     size_t s = 0;
     s += al256(sizeof(Traj<float>) * (size_t)B);
     s += al256(kMapBytes * 2 * (size_t)B);
     s += al256(sizeof(int4) * (size_t)total_items(cfgs, B));
     s += al256(sizeof(int) * (kMaxGrid + 1));
+    s += al256(sizeof(int2) * (size_t)total_pair_items(cfgs, B));
     return s;
 }
 
@@ -141,6 +151,23 @@ void lpt_schedule(const yy_batch* bt, int grid, int bn, std::vector<int4>& items
     start[grid] = (int)items.size();
 }
 
+// Items of the members on the float32 form, longest first: one block each, handed to the SMs
+// in this order, so that the long ones do not run on alone at the end.
+std::vector<int2> pair_schedule(const yy_batch* bt) {
+    std::vector<int> order;
+    for (int b = 0; b < bt->B; ++b)
+        if (bt->path[b] != 0) order.push_back(b);
+    auto cost = [&](int b) {
+        const yy_config& c = bt->filters[b]->cfg;
+        return (double)c.n * (c.r + 8.0);
+    };
+    std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return cost(x) > cost(y); });
+    std::vector<int2> items;
+    for (int b : order)
+        for (long long t = 0; t < pair_batch_blocks(bt->filters[b]->cfg.n); ++t) items.push_back(make_int2(b, (int)t));
+    return items;
+}
+
 // Builds and uploads the descriptors (trajectory constants and buffers, TMA maps, work
 // lists).  Synchronous; never called during stream capture.
 yy_status upload(yy_batch* bt) {
@@ -152,6 +179,7 @@ yy_status upload(yy_batch* bt) {
     std::vector<int> start, splits;
     lpt_schedule(bt, bt->grid, bt->bn, items, start, splits);
     if ((long long)items.size() > (long long)bt->max_items) return YY_ERR_ARG;
+    const std::vector<int2> pitems = pair_schedule(bt);
     for (int b = 0; b < bt->B; ++b) {
         yy_filter* f = bt->filters[b];
         tr[b].k = f->kf;
@@ -185,8 +213,12 @@ yy_status upload(yy_batch* bt) {
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(bt->d_cta_start, start.data(), sizeof(int) * start.size(), cudaMemcpyHostToDevice,
                             bt->stream);
+    if (e == cudaSuccess && !pitems.empty())
+        e = cudaMemcpyAsync(bt->d_pair_items, pitems.data(), sizeof(int2) * pitems.size(), cudaMemcpyHostToDevice,
+                            bt->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(bt->stream);
     if (e != cudaSuccess) return YY_ERR_CUDA;
+    bt->n_pair_items = (int)pitems.size();
     bt->n_items = (int)items.size();
     bt->n_tc = 0;
     for (int b = 0; b < bt->B; ++b) bt->n_tc += (bt->path[b] == 0);
@@ -203,7 +235,7 @@ yy_status batch_predict(yy_batch* bt) {
                                  bt->d_cta_start, bt->grid, bt->bn, bt->filters[0]->kf, bt->filters[0]->bf,
                                  bt->map_any, bt->stream, &l);
     if (e == cudaSuccess && bt->n_simt > 0)
-        e = launch_ksum_simt_batch<float>(bt->d_traj, bt->B, bt->N, bt->n_pad_max, bt->r_max, bt->stream, &l);
+        e = launch_pair_batch(bt->d_traj, bt->N, bt->d_pair_items, bt->n_pair_items, bt->stream, &l);
     bt->launches += l;
     return e == cudaSuccess ? YY_OK : YY_ERR_CUDA;
 }
@@ -277,6 +309,8 @@ yy_status yy_batch_create(const yy_config* cfgs, int32_t B, void* d_workspace, s
     p += al256(sizeof(int4) * (size_t)bt->max_items);
     bt->d_cta_start = reinterpret_cast<int*>(p);
     p += al256(sizeof(int) * (kMaxGrid + 1));
+    bt->d_pair_items = reinterpret_cast<int2*>(p);
+    p += al256(sizeof(int2) * (size_t)total_pair_items(cfgs, B));
     long long M = 0, H = 0;
     bt->r_max = 0;
     bt->n_pad_max = 0;

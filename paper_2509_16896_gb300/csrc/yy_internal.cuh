@@ -255,8 +255,8 @@ cudaError_t launch_ksum_tc_batch(const Traj<float>* d_traj, int B, int N, long l
                                  const int* d_cta_start, int grid, int bn, const Consts<float>& k_any,
                                  const Bufs<float>& b_any, const void* map_any, cudaStream_t s, int* launches);
 
-template <typename T>
-cudaError_t launch_ksum_simt_batch(const Traj<T>* d_traj, int B, int N, long long n_pad_max, int r_max,
-                                   cudaStream_t s, int* launches);
+long long pair_batch_blocks(long long n);
+cudaError_t launch_pair_batch(const Traj<float>* d_traj, int N, const int2* d_items, int n_items, cudaStream_t s,
+                              int* launches);
 
 }  // namespace yy

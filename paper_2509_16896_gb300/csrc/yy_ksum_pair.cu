@@ -113,6 +113,16 @@ __global__ void __launch_bounds__(THREADS, BLOCKS_PER_SM)
                           pair_smem);
 }
 
+// batched: block x processes item x = (member, target block)
+template <int N>
+__global__ void __launch_bounds__(THREADS, BLOCKS_PER_SM) kb_pair(const Traj<float>* __restrict__ tr,
+                                                                  const int2* __restrict__ items) {
+    extern __shared__ __align__(16) float pair_smem[];
+    const int2 it = items[blockIdx.x];
+    const Traj<float>& t = tr[it.x];
+    block<N, false, false>(t.k, t.b, (long long)it.y * BM, 0, 1, pair_smem);
+}
+
 // The skipping form: from this many coordinates (its reference pass and masks cost about 10 us,
 // and a tile is not given up before 64 coordinates: at r = 100 nothing is), up to this much
 // mask.  Measured, large-scale model at r = 1000, n = 2000, N = 2, full form 620 us per prediction:
@@ -141,6 +151,7 @@ cudaError_t set_attr_n() {
     cudaError_t e = cudaFuncSetAttribute(k_pair<N, false>, a, (int)smem_bytes<N, false, false>());
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_pair<N, true>, a, (int)smem_bytes<N, true, false>());
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_pair_skip<N>, a, (int)(smem_bytes<N, false, false, true>() + kMaxMaskBytes));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(kb_pair<N>, a, (int)smem_bytes<N, false, false>());
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_op_build<N>, a, (int)smem_bytes<N, false, true>());
     return e;
 }
@@ -253,6 +264,22 @@ cudaError_t launch_op_build(const Consts<float>& k, const Bufs<float>& b, bool f
         case 4: k_op_build<4><<<grid, THREADS, smem_bytes<4, false, true>(), s>>>(k, b, S, f); break;
         default: return cudaErrorInvalidValue;
     }
+    return cudaGetLastError();
+}
+
+long long pair_batch_blocks(long long n) { return (n + BM - 1) / BM; }
+
+cudaError_t launch_pair_batch(const Traj<float>* d_traj, int N, const int2* d_items, int n_items, cudaStream_t s,
+                              int* launches) {
+    if (n_items == 0) return cudaSuccess;
+    switch (N) {
+        case 1: kb_pair<1><<<n_items, THREADS, smem_bytes<1, false, false>(), s>>>(d_traj, d_items); break;
+        case 2: kb_pair<2><<<n_items, THREADS, smem_bytes<2, false, false>(), s>>>(d_traj, d_items); break;
+        case 3: kb_pair<3><<<n_items, THREADS, smem_bytes<3, false, false>(), s>>>(d_traj, d_items); break;
+        case 4: kb_pair<4><<<n_items, THREADS, smem_bytes<4, false, false>(), s>>>(d_traj, d_items); break;
+        default: return cudaErrorInvalidValue;
+    }
+    if (launches) *launches += 1;
     return cudaGetLastError();
 }
 

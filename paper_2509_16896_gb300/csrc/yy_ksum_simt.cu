@@ -1,6 +1,6 @@
-// Prediction step on the FMA pipes: the plain form in float64 (and in float32 for batches),
-// and the materialised operator's apply.  The plain float32 form of a single filter is in
-// yy_ksum_pair.cu, the screened one in yy_ksum_scr.cu.
+// Prediction step in float64 for long rows and noise coefficients, and the materialised
+// operator's apply.  The plain float32 form is in yy_ksum_pair.cu, the screened one in
+// yy_ksum_scr.cu, the float64 form of short rows in yy_ksum_f64.cu.
 //
 // For every target i and scale j (tau_j = dt / 2^(j-1)), in units relative to c_ref:
 //   L_j(i) - c_ref = (C_j - c_ref) - tau_j div f(x_i)
@@ -31,7 +31,6 @@ namespace {
 constexpr int BM = 64, BN = 64, BK = 16, TM = 4, TN = 4;
 
 template <typename T> __device__ __forceinline__ T exp_fast(T x);
-template <> __device__ __forceinline__ float exp_fast<float>(float x) { return exp2f(x * 1.4426950408889634f); }
 template <> __device__ __forceinline__ double exp_fast<double>(double x) { return exp(x); }
 }  // namespace
 
@@ -464,32 +463,6 @@ cudaError_t launch_op_apply(const Consts<float>& k, const Bufs<float>& b, cudaSt
     }
     return cudaGetLastError();
 }
-
-// batched: trajectory = blockIdx.y; blocks past a trajectory's rows return at once
-template <typename T, int N>
-__global__ void __launch_bounds__(256) kb_ksum_simt(const Traj<T>* __restrict__ tr) {
-    const Traj<T>& t = tr[blockIdx.y];
-    if (t.path == 0 || (long long)blockIdx.x * BM >= t.k.n_pad) return;
-    const int rk = ((t.k.r + BK - 1) / BK) * BK;
-    ksum_simt_body<T, N>(t.k, t.b, rk, blockIdx.x);
-}
-
-template <typename T>
-cudaError_t launch_ksum_simt_batch(const Traj<T>* d_traj, int B, int N, long long n_pad_max, int r_max,
-                                   cudaStream_t s, int* launches) {
-    (void)r_max;
-    const dim3 grid((unsigned)(n_pad_max / BM), B);
-    switch (N) {
-        case 1: kb_ksum_simt<T, 1><<<grid, 256, 0, s>>>(d_traj); break;
-        case 2: kb_ksum_simt<T, 2><<<grid, 256, 0, s>>>(d_traj); break;
-        case 3: kb_ksum_simt<T, 3><<<grid, 256, 0, s>>>(d_traj); break;
-        case 4: kb_ksum_simt<T, 4><<<grid, 256, 0, s>>>(d_traj); break;
-        default: return cudaErrorInvalidValue;
-    }
-    if (launches) *launches += 1;
-    return cudaGetLastError();
-}
-template cudaError_t launch_ksum_simt_batch<float>(const Traj<float>*, int, int, long long, int, cudaStream_t, int*);
 
 // Source ranges per target block of the plain form: enough blocks for two per SM (at most
 // kSimtMaxSplit ranges, none beyond the source tiles), when the filter has few target

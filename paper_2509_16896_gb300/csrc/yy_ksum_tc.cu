@@ -56,6 +56,7 @@
 
 #include "yy_combine.cuh"
 #include "yy_drift.cuh"
+#include "yy_pair_sums.cuh"
 #include "yy_tcgen05.cuh"
 
 namespace yy {
@@ -522,7 +523,11 @@ __device__ __forceinline__ float* part_slot(const Bufs<float>& b, long long i, i
 // (the odd CTA's arrive remotely).  Tiles to be screened again are the union of both
 // CTAs' marks.  Everything else -- screening, exact evaluation, row states -- is per CTA
 // and identical to the single-CTA kernel.
-template <int N, int BN, bool PAIR>
+// BATCH: the work list spans the filters of a batch (descriptors and TMA maps in global memory).
+// Only this instance takes the short rows' exact pairs through pair_sums_call: a call costs the
+// screening loop registers (with it the single filters' instances spilled: r = 100 prediction 90
+// -> 109 us, r = 1000 0.68 -> 0.81 ms), and it is batches that have many of them.
+template <int N, int BN, bool PAIR, bool BATCH>
 // One CTA per SM; with 10 warps two of the four SM sub-partitions hold three warps each, so
 // the register budget is 168 per thread.
 __global__ void __launch_bounds__(tc::NUM_THREADS, 1)
@@ -569,7 +574,7 @@ __global__ void __launch_bounds__(tc::NUM_THREADS, 1)
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const bool batched = (w.tr != nullptr);
+    constexpr bool batched = BATCH;
     const uint32_t rank = PAIR ? cluster_ctarank() : 0u;   // 0: even CTA (issues the MMAs)
     const int unit = PAIR ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;   // work list index
     const int it_begin = w.cta_start[unit];
@@ -1066,10 +1071,16 @@ __global__ void __launch_bounds__(tc::NUM_THREADS, 1)
                             const long long src = sb + c;
                             const float* us = b.u + (size_t)src * k.r_pad;
                             float s1 = 0.f, s2 = 0.f;
-                            for (int d = 0; d < k.r; ++d) {
-                                const float dl = ut[d] - us[d];
-                                s1 = fmaf(dl, dl, s1);
-                                s2 = fmaf(dl, drift_at(k, b, i, ut[d], d), s2);
+                            if (BATCH && b.store_f) {   // (loads a stage ahead instead of a word at a time)
+                                const float2 s12 = pair_sums_call(ut, b.f + (size_t)i * k.r_pad, us, k.r_pad);
+                                s1 = s12.x;
+                                s2 = s12.y;
+                            } else {
+                                for (int d = 0; d < k.r; ++d) {
+                                    const float dl = ut[d] - us[d];
+                                    s1 = fmaf(dl, dl, s1);
+                                    s2 = fmaf(dl, drift_at(k, b, i, ut[d], d), s2);
+                                }
                             }
                             add_score(s1, s2, src);
                             ++ncand;
@@ -1355,32 +1366,32 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
     return fn;
 }
 
-template <int BN, bool PAIR>
+template <int BN, bool PAIR, bool BATCH>
 cudaError_t set_attr_all() {
     cudaError_t e = cudaSuccess;
     const int sm = tc::Cfg<BN, PAIR>::SMEM_BYTES;
     // the block must be launchable at its size (registers per thread x threads)
     cudaFuncAttributes fa;
-    if ((e = cudaFuncGetAttributes(&fa, k_ksum_tc<3, BN, PAIR>)) != cudaSuccess) return e;
+    if ((e = cudaFuncGetAttributes(&fa, k_ksum_tc<3, BN, PAIR, BATCH>)) != cudaSuccess) return e;
     if (fa.maxThreadsPerBlock < tc::NUM_THREADS) return cudaErrorLaunchOutOfResources;
     const auto a = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_ksum_tc<1, BN, PAIR>, a, sm);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_ksum_tc<2, BN, PAIR>, a, sm);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_ksum_tc<3, BN, PAIR>, a, sm);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_ksum_tc<4, BN, PAIR>, a, sm);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_ksum_tc<1, BN, PAIR, BATCH>, a, sm);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_ksum_tc<2, BN, PAIR, BATCH>, a, sm);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_ksum_tc<3, BN, PAIR, BATCH>, a, sm);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_ksum_tc<4, BN, PAIR, BATCH>, a, sm);
     return e;
 }
 
-template <int BN>
+template <int BN, bool BATCH>
 cudaError_t launch_bn(int N, unsigned grid, const CUtensorMap& a, const CUtensorMap& bm, const Consts<float>& k,
                       const Bufs<float>& b, const TcWork& w, cudaStream_t s) {
     if (grid == 0) return cudaSuccess;
     const int sm = tc::Cfg<BN>::SMEM_BYTES;
     switch (N) {
-        case 1: k_ksum_tc<1, BN, false><<<grid, tc::NUM_THREADS, sm, s>>>(a, bm, k, b, w); break;
-        case 2: k_ksum_tc<2, BN, false><<<grid, tc::NUM_THREADS, sm, s>>>(a, bm, k, b, w); break;
-        case 3: k_ksum_tc<3, BN, false><<<grid, tc::NUM_THREADS, sm, s>>>(a, bm, k, b, w); break;
-        case 4: k_ksum_tc<4, BN, false><<<grid, tc::NUM_THREADS, sm, s>>>(a, bm, k, b, w); break;
+        case 1: k_ksum_tc<1, BN, false, BATCH><<<grid, tc::NUM_THREADS, sm, s>>>(a, bm, k, b, w); break;
+        case 2: k_ksum_tc<2, BN, false, BATCH><<<grid, tc::NUM_THREADS, sm, s>>>(a, bm, k, b, w); break;
+        case 3: k_ksum_tc<3, BN, false, BATCH><<<grid, tc::NUM_THREADS, sm, s>>>(a, bm, k, b, w); break;
+        case 4: k_ksum_tc<4, BN, false, BATCH><<<grid, tc::NUM_THREADS, sm, s>>>(a, bm, k, b, w); break;
         default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
@@ -1406,7 +1417,7 @@ cudaError_t launch_pair_n(unsigned clusters, const CUtensorMap& a, const Consts<
                           const TcWork& w, cudaStream_t s) {
     cudaLaunchAttribute at[1];
     const cudaLaunchConfig_t cfg = pair_config(clusters, s, at);
-    return cudaLaunchKernelEx(&cfg, k_ksum_tc<N, 256, true>, a, a, k, b, w);
+    return cudaLaunchKernelEx(&cfg, k_ksum_tc<N, 256, true, false>, a, a, k, b, w);
 }
 cudaError_t launch_pair(int N, unsigned clusters, const CUtensorMap& a, const Consts<float>& k, const Bufs<float>& b,
                         const TcWork& w, cudaStream_t s) {
@@ -1441,9 +1452,10 @@ bool make_tc_map(void* map_out, const void* base, long long rows, int cols, int 
 // when a BF16 handle or batch is created, so that no attribute call happens during
 // stream capture).
 cudaError_t prepare_ksum_tc() {
-    cudaError_t e = set_attr_all<256, false>();
-    if (e == cudaSuccess) e = set_attr_all<128, false>();
-    if (e == cudaSuccess) e = set_attr_all<256, true>();
+    cudaError_t e = set_attr_all<256, false, false>();
+    if (e == cudaSuccess) e = set_attr_all<256, true, false>();
+    if (e == cudaSuccess) e = set_attr_all<256, false, true>();
+    if (e == cudaSuccess) e = set_attr_all<128, false, true>();
     return e;
 }
 
@@ -1453,7 +1465,7 @@ int tc_pair_max_clusters() {
     cudaLaunchAttribute at[1];
     const cudaLaunchConfig_t cfg = pair_config(1, nullptr, at);
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, k_ksum_tc<3, 256, true>, &cfg) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveClusters(&n, k_ksum_tc<3, 256, true, false>, &cfg) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }
@@ -1479,7 +1491,7 @@ cudaError_t launch_ksum_tc(const Consts<float>& k, const Bufs<float>& b, cudaStr
     const TcWork w{nullptr, nullptr, b.tc_items, b.tc_cta_start, 1, k.wait_ns};
     // tc_grid counts CTAs; a paired schedule has tc_grid / 2 work lists, one per cluster
     e = b.tc_pair ? launch_pair(k.N, (unsigned)(b.tc_grid / 2), ma, k, b, w, s)
-                  : launch_bn<256>(k.N, (unsigned)b.tc_grid, ma, mb, k, b, w, s);
+                  : launch_bn<256, false>(k.N, (unsigned)b.tc_grid, ma, mb, k, b, w, s);
     if (e != cudaSuccess) return e;
     int l = k.tc_sym ? 3 : 2;
     if (b.tc_splits > 1 || k.tc_sym) {
@@ -1507,8 +1519,8 @@ cudaError_t launch_ksum_tc_batch(const Traj<float>* d_traj, int B, int N, long l
     if (e != cudaSuccess) return e;
     const CUtensorMap& map_any = *static_cast<const CUtensorMap*>(map_any_v);
     const TcWork w{d_traj, static_cast<const CUtensorMap*>(d_maps), d_items, d_cta_start, B, k_any.wait_ns};
-    e = (bn == 128) ? launch_bn<128>(N, (unsigned)grid, map_any, map_any, k_any, b_any, w, s)
-                    : launch_bn<256>(N, (unsigned)grid, map_any, map_any, k_any, b_any, w, s);
+    e = (bn == 128) ? launch_bn<128, true>(N, (unsigned)grid, map_any, map_any, k_any, b_any, w, s)
+                    : launch_bn<256, true>(N, (unsigned)grid, map_any, map_any, k_any, b_any, w, s);
     if (e != cudaSuccess) return e;
     const dim3 mg((unsigned)std::min<long long>((n_pad_max + 255) / 256, 256), B);
     switch (N) {

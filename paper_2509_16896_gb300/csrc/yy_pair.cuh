@@ -30,6 +30,7 @@
 #pragma once
 
 #include "yy_combine.cuh"
+#include "yy_pair_sums.cuh"
 #include "yy_tcgen05.cuh"
 
 namespace yy {
@@ -111,40 +112,6 @@ __device__ __forceinline__ float max_nan(float a, float b) {
 constexpr float kZeroGap = 105.0f;
 
 constexpr int kThinGroups = 2;
-// S1 and S2 of one pair over all coordinates in increasing order, loads a stage ahead.
-__device__ __forceinline__ void pair_sums_thread(const float* __restrict__ ut, const float* __restrict__ ft,
-                                                 const float* __restrict__ us, int r_pad, float& s1, float& s2) {
-    constexpr int Q = 4;   // float4 per stage and operand
-    float4 a[Q], f[Q], c[Q];
-    auto get = [&](int d) {
-#pragma unroll
-        for (int q = 0; q < Q; ++q) {
-            a[q] = *reinterpret_cast<const float4*>(ut + d + 4 * q);
-            f[q] = *reinterpret_cast<const float4*>(ft + d + 4 * q);
-            c[q] = *reinterpret_cast<const float4*>(us + d + 4 * q);
-        }
-    };
-    s1 = s2 = 0.f;
-    get(0);
-    for (int d = 0; d < r_pad; d += 4 * Q) {   // padded coordinates are zero in all three
-        float4 x[Q], y[Q], z[Q];
-#pragma unroll
-        for (int q = 0; q < Q; ++q) { x[q] = a[q]; y[q] = f[q]; z[q] = c[q]; }
-        if (d + 4 * Q < r_pad) get(d + 4 * Q);
-#pragma unroll
-        for (int q = 0; q < Q; ++q) {
-            const float xs[4] = {x[q].x, x[q].y, x[q].z, x[q].w}, ys[4] = {y[q].x, y[q].y, y[q].z, y[q].w};
-            const float zs[4] = {z[q].x, z[q].y, z[q].z, z[q].w};
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const float dl = xs[e] - zs[e];
-                s1 = fmaf(dl, dl, s1);
-                s2 = fmaf(dl, ys[e], s2);
-            }
-        }
-    }
-}
-
 // One block: targets i0 .. i0 + BM - 1 against the groups of 64 sources in the range [split /
 // nsplit, (split + 1) / nsplit), TN / 4 groups per source tile.  nsplit > 1: the rows' (max,
 // sum) go to b.simt_part and a merge kernel applies the combination.  OP: every pair's score
