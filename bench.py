@@ -41,7 +41,7 @@ DEFAULT_WORKLOAD = "cubic_r1000_n65536"
 # kernel, from one ncu capture of the workload, keyed by workload, screen operands and
 # whether the kernel ran on CTA pairs.  An entry is removed whenever the kernel changes
 # after its capture.
-NCU_TRAFFIC = {("cubic_r1000_n65536", "fp8", False): 39.310848e6 + 0.567552e6}
+NCU_TRAFFIC = {}
 # --cta-pair: the tensor-core prediction on 2-CTA clusters (yy_set_cta_pair)
 CTA_PAIR = False
 METRIC = "filter steps/s & kernel pair-evals/s at r=1000: mixed vs FP32, same RMSE"
@@ -286,7 +286,7 @@ def measure_single(w, prec, screen_type, screen_prefix, K, W, device, seed, dist
     else:
         flops = 3.0 * w.n * w.n * w.r
         roof = {"bound": "alu", "achieved": round(flops / (pred_ms / 1e3) / 1e12, 3), "peak": _fma_peak(),
-                "unit": "TFLOP/s", "kernel": "k_ksum_simt (difference form)", "kernel_ms": round(pred_ms, 4),
+                "unit": "TFLOP/s", "kernel": "k_pair / k_pair_skip (difference form)", "kernel_ms": round(pred_ms, 4),
                 "algorithmic_flops_per_launch": flops,
                 "peak_source": "derived: 152 SMs x 128 FP32 lanes x 2 flops x max SM clock"}
     roof["frac"] = round(roof["achieved"] / roof["peak"], 4)
@@ -330,7 +330,7 @@ def _time_precision(w, prec, steps, warmup, tr, device, screen_prefix=0):
 
 
 def _comparators(w, K, W, tr, device, fp32_steps, est):
-    """The plain FP32 GPU form (every pair, difference form) and the screened FP32 form
+    """The plain FP32 GPU form (difference form) and the screened FP32 form
     (the same kind of screen with its bound on the FMA pipes), each with its RMSE next to
     the mixed path's on the same steps: the first isolates pruning + precision, the second
     precision alone."""

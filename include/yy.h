@@ -87,9 +87,9 @@ typedef enum { YY_NODES_SOBOL = 0, YY_NODES_HALTON = 1, YY_NODES_FAURE = 2 } yy_
  * float32 next to the largest of its row is not summed to the end).  BF16: a tcgen05 BF16 Gram product screens out pairs
  * whose kernel term is provably negligible, and the remaining pairs are evaluated exactly
  * in float32 (results agree with FP32 within float32 rounding).  FP32_SCREEN: the same kind
- * of screen on the FMA pipes, no tensor cores: a tile of 64 x 64 pairs is skipped when the
- * exact float32 squared distance of every live pair over the first 64 k coordinates
- * (k = screen_prefix, default half of the 64-coordinate chunks) exceeds the row's screening
+ * of screen on the FMA pipes, no tensor cores: a tile of pairs is skipped when a lower bound of
+ * every live pair's squared distance over the first 64 k coordinates (k = screen_prefix,
+ * default half of the 64-coordinate chunks; r < 128: no screen) exceeds the row's screening
  * radius; every other tile is evaluated exactly as in FP32 (results agree with FP32 within
  * float32 rounding).  Not accepted by batches. */
 typedef enum { YY_PREC_FP64 = 0, YY_PREC_FP32 = 1, YY_PREC_BF16 = 2, YY_PREC_FP32_SCREEN = 3 } yy_precision;
@@ -472,7 +472,7 @@ YY_EXPORT yy_status yy_tune_materialise(yy_filter* f, int32_t predicts_per_build
 
 /* Routing of a BF16 filter's prediction (no counterpart in the paper; the paper evaluates
  * every pair): the screened tensor-core form of yy_predict, or the plain float32 form of
- * YY_PREC_FP32 (every pair, same results within float32 rounding).  The screen wins where
+ * YY_PREC_FP32 (same results within float32 rounding).  The screen wins where
  * it proves most pairs negligible; where the weights spread over many nats (the paper's
  * large-scale workload) nearly every pair survives it and the plain form is faster.
  * yy_set_route: plain = 1 routes to the plain form, 0 back to the screen (the default).
