@@ -348,7 +348,10 @@ YY_EXPORT yy_status yy_batch_run_steps(yy_batch* bt, const double* d_dy_all, int
 YY_EXPORT yy_status yy_batch_predict(yy_batch* bt);
 
 /* Captures yy_batch_run_steps(bt, d_dy_all, K, d_hist) as a CUDA graph (needs a created
- * stream); yy_batch_graph_launch replays it. */
+ * stream); yy_batch_graph_launch replays it.  After a change of schedule or routing has taken
+ * effect (with the next yy_batch_predict, yy_batch_run_steps or yy_batch_autotune) the replay
+ * follows it: where it changes the launches, yy_batch_graph_launch first captures the steps
+ * again on the same buffers. */
 YY_EXPORT yy_status yy_batch_graph_capture(yy_batch* bt, const double* d_dy_all, int64_t K, double* d_hist);
 YY_EXPORT yy_status yy_batch_graph_launch(yy_batch* bt);
 

@@ -44,6 +44,7 @@ struct yy_batch {
     int n_pair_items;
     // schedule
     int bn, grid, n_items;
+    int bn_up, grid_up;             // the schedule the uploaded work lists were built for
     std::vector<int> path;          // per filter: 0 = tcgen05 screen, 1 = FP32 form
     double dense_frac;              // screen pass fraction above which a filter is routed to FP32
     int n_tc, n_simt;
@@ -52,6 +53,12 @@ struct yy_batch {
     cudaGraph_t graph;
     cudaGraphExec_t gexec;
     long long graph_kernels;
+    // what the graph was captured with: its buffers, and the launch shapes that upload() derives
+    // from the schedule and the routing (the rest of the descriptors is read on the device)
+    const double* graph_dy;
+    long long graph_K;
+    double* graph_hist;
+    int graph_bn, graph_grid, graph_n_tc, graph_n_pair;
     alignas(64) unsigned char map_any[128];
 };
 
@@ -168,6 +175,12 @@ std::vector<int2> pair_schedule(const yy_batch* bt) {
     return items;
 }
 
+// The captured launches cover the work lists that are on the device now.
+bool graph_current(const yy_batch* bt) {
+    return bt->graph_bn == bt->bn_up && bt->graph_grid == bt->grid_up && bt->graph_n_pair == bt->n_pair_items &&
+           (bt->graph_n_tc > 0) == (bt->n_tc > 0);
+}
+
 // Builds and uploads the descriptors (trajectory constants and buffers, TMA maps, work
 // lists).  Synchronous; never called during stream capture.
 yy_status upload(yy_batch* bt) {
@@ -220,6 +233,8 @@ yy_status upload(yy_batch* bt) {
     if (e != cudaSuccess) return YY_ERR_CUDA;
     bt->n_pair_items = (int)pitems.size();
     bt->n_items = (int)items.size();
+    bt->bn_up = bt->bn;
+    bt->grid_up = bt->grid;
     bt->n_tc = 0;
     for (int b = 0; b < bt->B; ++b) bt->n_tc += (bt->path[b] == 0);
     bt->n_simt = bt->B - bt->n_tc;
@@ -428,12 +443,25 @@ yy_status yy_batch_graph_capture(yy_batch* bt, const double* d_dy_all, int64_t K
     if (e != cudaSuccess) { cudaGraphDestroy(g); return YY_ERR_CUDA; }
     bt->graph = g;
     bt->gexec = ex;
+    bt->graph_dy = d_dy_all;
+    bt->graph_K = K;
+    bt->graph_hist = d_hist;
+    bt->graph_bn = bt->bn_up;
+    bt->graph_grid = bt->grid_up;
+    bt->graph_n_tc = bt->n_tc;
+    bt->graph_n_pair = bt->n_pair_items;
     return YY_OK;
 }
 
 yy_status yy_batch_graph_launch(yy_batch* bt) {
     if (!bt) return YY_ERR_ARG;
     if (!bt->gexec) return YY_ERR_STATE;
+    // a schedule or routing that was uploaded since gives the launches other sizes: capture again
+    // (on the same buffers), or members would be left without a prediction
+    if (!graph_current(bt)) {
+        const yy_status st = yy_batch_graph_capture(bt, bt->graph_dy, bt->graph_K, bt->graph_hist);
+        if (st != YY_OK) return st;
+    }
     bt->launches += bt->graph_kernels;
     return cudaGraphLaunch(bt->gexec, bt->stream) == cudaSuccess ? YY_OK : YY_ERR_CUDA;
 }

@@ -119,3 +119,41 @@ def test_every_schedule_gives_the_same_prediction(yy_lib, tmp_path):
     torch.cuda.synchronize()
     h = hist.cpu().numpy()
     assert np.max(np.abs(h - ref) / np.maximum(1.0, np.abs(ref))) <= 1e-5
+
+
+@pytest.mark.parametrize("before,after,sched", [([0, 1, 0, 1, 1, 0], [1, 1, 1, 1, 1, 0], None),
+                                                ([1, 1, 0, 1, 1, 0], [0, 0, 0, 1, 0, 0], None),
+                                                ([0] * 6, [0, 1, 0, 0, 1, 0], None),
+                                                ([1] * 6, [0, 1, 0, 0, 1, 0], None),
+                                                ([0, 1] * 3, [1, 0] * 3, (128, 40))])
+def test_graph_replay_follows_a_new_routing(yy_lib, before, after, sched):
+    """Members moved between the screen and the float32 form, and the schedule changed, after a
+    capture: the replay advances every member as run_steps with the new routing does (same bar
+    as between schedules)."""
+    import torch
+    K = 3
+    _, dy_all = _inputs(K)
+    a = _batch("bf16")
+    a.set_routing(after)
+    ha = torch.zeros((K, a.H), dtype=torch.float64, device="cuda")
+    a.run_steps(dy_all, ha)
+    g = _batch("bf16")
+    g.set_routing(before)
+    hg = torch.zeros((K, g.H), dtype=torch.float64, device="cuda")
+    g.graph_capture(dy_all, hg)
+    g.graph_launch()
+    g.set_routing(after)
+    if sched:
+        g.set_schedule(*sched)
+    g.predict()   # the new routing takes effect
+    for b, (m, r, n, s) in enumerate(MEMBERS):
+        poly, scr = sobol_inputs(r, s)
+        g.filters[b].init_nodes(poly, scr, np.zeros(r))
+    hg.zero_()
+    torch.cuda.synchronize()
+    g.graph_launch()
+    torch.cuda.synchronize()
+    h, ref = hg.cpu().numpy(), ha.cpu().numpy()
+    for b in range(len(MEMBERS)):
+        hb, rb = (x[:, g.hist_off[b]:g.hist_off[b + 1]] for x in (h, ref))
+        assert np.max(np.abs(hb - rb) / np.maximum(1.0, np.abs(rb))) <= 1e-6, b
