@@ -6,14 +6,17 @@
 // next to its largest, so each pair is first scored in float32 (the coordinates are float32
 // numbers; 64 times the rate) and only pairs that can carry more than e^-(ln n + 40) of their
 // row's largest term are evaluated in float64: everything dropped from a row adds up to less
-// than e^-40, a thirtieth of a unit in the last place.  The float32 score is compared with
-// a margin of 1 + 1e-5 times the magnitudes that enter it, its rounding being below 1e-6 of them.
+// than e^-40, a thirtieth of a unit in the last place.  Both sides of the comparison carry the
+// bound of their float32 rounding (kErr): a pair's score its upper, the row's largest its lower.
 //
 // One warp per target row.  A block's eight warps share tiles of sources staged in shared
 // memory; a warp scores the tile in float32 twice, for the largest score (the reference of the
-// log-sum-exp and of the selection; close to the maximum is all it has to be) and for the
+// selection, and of the log-sum-exp: close below the maximum is all it has to be) and for the
 // survivors, which it queues and then evaluates 32 at a time, one per lane, with one exponential
-// per scale and no comparison in float64.  The lanes' sums are added at the end, and the eight
+// per scale and no comparison in float64.  Where a survivor's magnitudes are so large that its
+// float32 score is off by more than kMaxErr nats (weights spread over 1e8 nats, a step far
+// shorter than the box is wide), e^(score - reference) could overflow, and the tile's
+// reference is the largest of the survivors' float64 scores, evaluated once more.  The lanes' sums are added at the end, and the eight
 // rows' combinations are taken side by side by eight lanes.  Measured at r = 2, n = 1024, N = 2
 // (box 8 wide): every pair in float64, coordinates padded to 16: 370 us; selection against
 // the row's own term: 62 us (a row far from the posterior's peak keeps a third of the
@@ -29,6 +32,10 @@ namespace {
 constexpr int kRows = 8;          // target rows (warps) per block
 constexpr int kTileFloats = 4096; // coordinates of one source tile in shared memory, at most
 constexpr int kTileMax = 1024;    // sources of one tile, at most
+// A float32 score of at most 64 coordinates is off by less than kErr times the magnitudes that
+// enter it (two chains of 64 FMAs, 3.9e-6, and the roundings of the operands).
+constexpr float kErr = 1e-5f;
+constexpr float kMaxErr = 100.0f;  // up to here a float32 bound serves as the sums' reference
 
 __device__ __forceinline__ int tile_sources(int r) { return min(kTileMax, kTileFloats / (r + 1) / 32 * 32); }
 
@@ -46,8 +53,8 @@ __global__ void __launch_bounds__(32 * kRows, 1)
     const long long i = k.row0 + (long long)blockIdx.x * kRows + w;
     const bool target = i < k.row1 && i < k.n && !b.mask[i];
     const double* fi = b.f + (size_t)i * k.r_pad;
-    double rowc[N], sm[N];
-    float top[N];   // reference of the sums
+    double rowc[N], sm[N], ref[N];   // sums of e^(score - ref)
+    float top[N];                    // lower bounds of the row's largest score
     const double nf = target ? b.nf[i] : 0.0;
     if (target)
         for (int d = lane; d < r; d += 32) {
@@ -55,7 +62,7 @@ __global__ void __launch_bounds__(32 * kRows, 1)
             ff[w][d] = (float)fi[d];
         }
     __syncwarp();
-    const float gap = logf((float)k.n) + 40.0f;
+    const float gap = logf((float)k.n) + 41.0f;
     float rowf[N], i2t[N];
 #pragma unroll
     for (int j = 0; j < N; ++j) {
@@ -63,6 +70,7 @@ __global__ void __launch_bounds__(32 * kRows, 1)
         rowf[j] = (float)rowc[j];
         i2t[j] = (float)k.inv2tau[j];
         sm[j] = 0.0;
+        ref[j] = -INFINITY;
         top[j] = -INFINITY;
     }
     for (long long s0 = 0; s0 < k.n; s0 += TS) {
@@ -81,8 +89,8 @@ __global__ void __launch_bounds__(32 * kRows, 1)
         }
         __syncthreads();
         if (!target) continue;
-        // float32 scores of source s of the tile; *mag: the magnitudes that enter them
-        auto scores = [&](int s, float ls, float (&sc)[N], float* mag) {
+        // float32 scores of source s of the tile; *err: a bound of their rounding
+        auto scores = [&](int s, float ls, float (&sc)[N], float* err) {
             const float* p = us + s * rs;
             float s1 = 0.f, s2 = 0.f, a2 = 0.f;
             for (int d = 0; d < r; ++d) {
@@ -97,41 +105,39 @@ __global__ void __launch_bounds__(32 * kRows, 1)
                 sc[j] = fmaf(-s1, i2t[j], s2) + (rowf[j] + ls);
                 m = fmaxf(m, fmaf(s1, i2t[j], a2 + fabsf(ls) + fabsf(rowf[j])));
             }
-            *mag = m;
+            *err = kErr * m;
         };
-        // 1. the tile's largest score per scale, into the reference
+        // 1. a lower bound of the tile's largest score per scale (an undefined one bounds nothing)
         float fm[N];
 #pragma unroll
         for (int j = 0; j < N; ++j) fm[j] = -INFINITY;
         for (int s = lane; s < ts; s += 32) {
             const float ls = lsf[s];
             if (ls == -INFINITY) continue;
-            float sc[N], mag;
-            scores(s, ls, sc, &mag);
+            float sc[N], err;
+            scores(s, ls, sc, &err);
 #pragma unroll
-            for (int j = 0; j < N; ++j) fm[j] = fmaxf(fm[j], sc[j]);
+            for (int j = 0; j < N; ++j) fm[j] = fmaxf(fm[j], sc[j] - err);
         }
 #pragma unroll
         for (int j = 0; j < N; ++j) {
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) fm[j] = fmaxf(fm[j], __shfl_xor_sync(0xffffffffu, fm[j], o));
-            if (fm[j] > top[j]) {
-                if (top[j] != -INFINITY) sm[j] *= exp((double)top[j] - (double)fm[j]);
-                top[j] = fm[j];
-            }
+            top[j] = fmaxf(top[j], fm[j]);
         }
-        // 2. the sources that can count next to it
+        // 2. the sources that can count next to it (an undefined score is kept)
         int nq = 0;
+        bool exact_ref = false;
         for (int c = 0; c < ts; c += 32) {
             const int s = c + lane;
             bool keep = false;
             const float ls = s < ts ? lsf[s] : -INFINITY;
             if (ls != -INFINITY) {
-                float sc[N], mag;
-                scores(s, ls, sc, &mag);
+                float sc[N], err;
+                scores(s, ls, sc, &err);
 #pragma unroll
-                for (int j = 0; j < N; ++j)
-                    keep |= !(sc[j] < top[j] - gap - (1.f + 1e-5f * (mag + fabsf(top[j]))));
+                for (int j = 0; j < N; ++j) keep |= !(sc[j] + err < top[j] - gap);
+                exact_ref |= keep && !(err < kMaxErr);
             }
             const uint32_t bal = __ballot_sync(0xffffffffu, keep);
             if (keep) queue[w][nq + __popc(bal & ((1u << lane) - 1u))] = (unsigned short)s;
@@ -139,9 +145,8 @@ __global__ void __launch_bounds__(32 * kRows, 1)
         }
         __syncwarp();
         // 3. their terms, in float64
-        for (int q0 = 0; q0 < nq; q0 += 32) {
-            const bool on = q0 + lane < nq;
-            const int s = on ? queue[w][q0 + lane] : 0;
+        auto scores64 = [&](int q, double (&sc)[N]) {
+            const int s = q < nq ? queue[w][q] : 0;
             const float* p = us + s * rs;
             double s1 = 0.0, s2 = 0.0;
             for (int d = 0; d < r; ++d) {
@@ -149,12 +154,41 @@ __global__ void __launch_bounds__(32 * kRows, 1)
                 s1 = fma(dl, dl, s1);
                 s2 = fma(dl, fi[d], s2);
             }
-            const double ls = on ? b.logw[s0 + s] : -INFINITY;
+            const double ls = q < nq ? b.logw[s0 + s] : -INFINITY;
+#pragma unroll
+            for (int j = 0; j < N; ++j) sc[j] = fma(-s1, k.inv2tau[j], s2) + (rowc[j] + ls);
+        };
+        double tref[N];   // the tile's reference
+#pragma unroll
+        for (int j = 0; j < N; ++j) tref[j] = (double)fm[j];
+        if (__any_sync(0xffffffffu, exact_ref)) {
+#pragma unroll
+            for (int j = 0; j < N; ++j) tref[j] = -INFINITY;
+            for (int q0 = 0; q0 < nq; q0 += 32) {
+                double sc[N];
+                scores64(q0 + lane, sc);
+#pragma unroll
+                for (int j = 0; j < N; ++j) tref[j] = fmax(tref[j], sc[j]);
+            }
+#pragma unroll
+            for (int j = 0; j < N; ++j)
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) tref[j] = fmax(tref[j], __shfl_xor_sync(0xffffffffu, tref[j], o));
+        }
+#pragma unroll
+        for (int j = 0; j < N; ++j)
+            if (tref[j] > ref[j]) {
+                if (ref[j] != -INFINITY) sm[j] *= exp(ref[j] - tref[j]);
+                ref[j] = tref[j];
+            }
+        for (int q0 = 0; q0 < nq; q0 += 32) {
+            const bool on = q0 + lane < nq;
             double e[N];
+            scores64(q0 + lane, e);
 #pragma unroll
-            for (int j = 0; j < N; ++j) e[j] = exp(fma(-s1, k.inv2tau[j], s2) + (rowc[j] + ls) - (double)top[j]);
+            for (int j = 0; j < N; ++j) e[j] = exp(e[j] - ref[j]);
 #pragma unroll
-            for (int j = 0; j < N; ++j) sm[j] += on ? e[j] : 0.0;
+            for (int j = 0; j < N; ++j) sm[j] += on && ref[j] != -INFINITY ? e[j] : 0.0;
         }
         __syncwarp();
     }
@@ -163,7 +197,7 @@ __global__ void __launch_bounds__(32 * kRows, 1)
         for (int j = 0; j < N; ++j) {
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) sm[j] += __shfl_xor_sync(0xffffffffu, sm[j], o);
-            if (lane == 0) { smx[w][j] = (double)top[j]; ssm[w][j] = sm[j]; }
+            if (lane == 0) { smx[w][j] = ref[j]; ssm[w][j] = sm[j]; }
         }
     }
     __syncthreads();

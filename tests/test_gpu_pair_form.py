@@ -117,3 +117,35 @@ def test_float64_short_rows(yy_lib, r, n, N, R, spread):
     assert both.mean() >= 0.99, np.nonzero(~both)[0][:5]
     ok, _ = combination_err_ok(got[both], ref[both], Lj[both], p.coef, lw[both], 1e-10, eps=2.0 ** -53)
     assert ok
+
+
+@pytest.mark.parametrize("r,n,N", [(1, 100, 1), (2, 1500, 3), (9, 300, 1), (33, 200, 3), (64, 150, 1)])
+@pytest.mark.parametrize("kind", ["weights", "distances", "both"])
+def test_float64_short_rows_large_magnitudes(yy_lib, kind, r, n, N):
+    """Scores far beyond float32's resolution of a nat: log-weights of 3e11 and more nats, and
+    distances of 1e12 nats between the nodes (a step much shorter than the box), where a row
+    without weight of its own has no near source.  Against the oracle within the float64 bar."""
+    from oracle import filter as F
+    from paper_2509_16896_gb300 import binding
+    dt = 0.01 if kind == "weights" else 1e-13
+    f = binding.Filter(binding.make_config(model="cubic", r=r, n=n, dt=dt, R=1.0, n_scales=N, precision="f64"))
+    poly, scr = sobol_inputs(r, 70 + r)
+    f.init_nodes(poly, scr, np.zeros(r))
+    u, _ = f.get_nodes()
+    p = oracle_problem("cubic", r, n, dt, 1.0, N)
+    rng = np.random.default_rng(1000 * r + n)
+    lw = -2.0 * rng.random(n) if kind == "distances" else -1e11 * (3.0 + rng.random(n))
+    lw[rng.random(n) < 0.5] = -np.inf
+    lw[n // 3] = 0.0 if kind == "distances" else -3e11 - 12345.678
+    centre = rng.standard_normal(r)
+    f.set_state(centre, lw, 0.0, 1)
+    f.predict()
+    pred, off = f.get_log_weights()
+    prep = F.prepare(p, u, centre)
+    Lj = F.kernel_lse(p, prep, lw)
+    ref, _ = F.combine(p, Lj, lw, prep.mask)
+    got = pred + off
+    both = np.isfinite(got) == np.isfinite(ref)
+    assert both.mean() >= 0.99, np.nonzero(~both)[0][:5]
+    ok, _ = combination_err_ok(got[both], ref[both], Lj[both], p.coef, lw[both], 1e-10, eps=2.0 ** -53)
+    assert ok
