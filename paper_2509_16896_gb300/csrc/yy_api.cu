@@ -477,7 +477,7 @@ yy_status yy_create(const yy_config* cfg, void* d_workspace, size_t bytes, void*
     else carve<float>(cfg, f->ws, &f->bf);
     cudaError_t e = cudaSuccess;
     if (cfg->precision == YY_PREC_BF16) e = prepare_ksum_tc();
-    if (e == cudaSuccess && !f->fp64) e = prepare_pair();
+    if (e == cudaSuccess) e = f->fp64 ? prepare_ksum_f64() : prepare_pair();
     if (e == cudaSuccess && cfg->materialise && !f->fp64) e = prepare_op_apply();
     if (e == cudaSuccess) e = cudaMemsetAsync(d_workspace, 0, need, f->stream);
     if (e != cudaSuccess) { delete f; return YY_ERR_CUDA; }

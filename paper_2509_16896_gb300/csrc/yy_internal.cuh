@@ -192,6 +192,7 @@ cudaError_t launch_prep(const Consts<T>& k, const Bufs<T>& b, bool init_weights,
 
 cudaError_t launch_ksum_simt(const Consts<double>& k, const Bufs<double>& b, cudaStream_t s, int* launches = nullptr);
 bool ksum_f64_fits(const Consts<double>& k);
+cudaError_t prepare_ksum_f64();
 cudaError_t launch_ksum_f64(const Consts<double>& k, const Bufs<double>& b, cudaStream_t s, int* launches);
 cudaError_t launch_pair(const Consts<float>& k, const Bufs<float>& b, cudaStream_t s, int* launches);
 cudaError_t prepare_pair();

@@ -149,3 +149,11 @@ def test_float64_short_rows_large_magnitudes(yy_lib, kind, r, n, N):
     assert both.mean() >= 0.99, np.nonzero(~both)[0][:5]
     ok, _ = combination_err_ok(got[both], ref[both], Lj[both], p.coef, lw[both], 1e-10, eps=2.0 ** -53)
     assert ok
+
+
+@pytest.mark.parametrize("r,n,N,R", [(1, 1025, 2, 2.0), (1, 2100, 1, 5.0), (7, 1800, 3, 1.0), (31, 600, 2, 0.3),
+                                     (48, 353, 4, 0.05), (64, 129, 2, 0.05)])
+def test_float64_short_rows_source_tiles(yy_lib, r, n, N, R):
+    """Several source tiles, the last one ragged (a tile holds 1024 sources of short rows, 128 of
+    64 coordinates), from boxes with few pairs in reach to boxes with all of them."""
+    test_float64_short_rows(yy_lib, r, n, N, R, 2.0)
