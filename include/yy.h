@@ -89,7 +89,8 @@ typedef enum { YY_NODES_SOBOL = 0, YY_NODES_HALTON = 1, YY_NODES_FAURE = 2 } yy_
  * in float32 (results agree with FP32 within float32 rounding).  FP32_SCREEN: the same kind
  * of screen on the FMA pipes, no tensor cores: a tile of pairs is skipped when a lower bound of
  * every live pair's squared distance over the first 64 k coordinates (k = screen_prefix,
- * default half of the 64-coordinate chunks; r < 128: no screen) exceeds the row's screening
+ * default half of the 64-coordinate chunks; no screen where it cannot pay: r < 64, or r < 128
+ * with n < 4096) exceeds the row's screening
  * radius; every other tile is evaluated exactly as in FP32 (results agree with FP32 within
  * float32 rounding).  Not accepted by batches. */
 typedef enum { YY_PREC_FP64 = 0, YY_PREC_FP32 = 1, YY_PREC_BF16 = 2, YY_PREC_FP32_SCREEN = 3 } yy_precision;

@@ -184,13 +184,21 @@ __global__ void __launch_bounds__(THREADS, 4)
 
 }  // namespace
 
+// Where the screen runs.  Below 64 coordinates the plain form is as fast as a screen that drops
+// everything but needs 64 coordinates to see it was before the packed loops (r = 64, n = 16384, N = 2:
+// 2.35 ms against 2.2 ms plain), and with few targets its passes cost more than they
+// save.  Measured at N = 2, us, plain form -> screen where no pair is left / every tile is left:
+// r = 64 n = 2048 60 -> 58 / 68, n = 4096 193 -> 82 / 107; r = 100 n = 2048 79 -> 67 / 118, n = 4096 277 -> 93 /
+// 304, n = 16384 3280 -> 511 / 4088; r = 127 n = 4096 331 -> 81 / 329, n = 16384 3989 -> 496 / 3826.
+// Longer rows are screened at any size: their tiles are also given up on the way.
+static bool screen_pays(const Consts<float>& k) { return k.r >= 128 || (k.r >= 64 && k.n >= 4096); }
+
 size_t scr_flag_words(long long n_pad) { return (size_t)(n_pad / 32) * (size_t)((n_pad / 128 + 31) / 32); }
 
 // First pass over at most k1 coordinates (a multiple of 64: the norms come in chunks of 64),
 // then exact evaluation of every flagged tile.
 cudaError_t launch_ksum_scr32(const Consts<float>& k, const Bufs<float>& b, int k1, cudaStream_t s, int* launches) {
-    // short rows leave the screen nothing to drop: the plain form
-    if (k.r < 128 || !pair_skip_fits(k, b)) return launch_pair(k, b, s, launches);
+    if (!screen_pays(k) || !pair_skip_fits(k, b)) return launch_pair(k, b, s, launches);
     if (!b.nu_chunk || !b.scr_flags) return cudaErrorInvalidValue;
     k1 = std::max(64, std::min((k1 + 63) / 64 * 64, k.r_pad));
     const float T = logf((float)k.n) + 20.0f;

@@ -157,3 +157,37 @@ def test_float64_short_rows_source_tiles(yy_lib, r, n, N, R):
     """Several source tiles, the last one ragged (a tile holds 1024 sources of short rows, 128 of
     64 coordinates), from boxes with few pairs in reach to boxes with all of them."""
     test_float64_short_rows(yy_lib, r, n, N, R, 2.0)
+
+
+@pytest.mark.parametrize("r,n,N,R,spread", [(64, 4096, 1, 1.0, 2.0), (65, 4100, 2, 0.3, 60.0), (100, 4500, 2, 0.3, 2.0),
+                                            (100, 5000, 3, 0.1, 2.0), (127, 4097, 4, 1.0, 3000.0)])
+def test_float32_screen_of_mid_rows(yy_lib, r, n, N, R, spread):
+    """The float32 screen below 128 coordinates, from boxes in which nearly every pair drops out to
+    boxes in which none does: the screen is what runs (its launches, at least three), and the
+    predictions are the oracle's within the float32 bar."""
+    from oracle import filter as F
+    from paper_2509_16896_gb300 import binding
+    f = binding.Filter(binding.make_config(model="cubic", r=r, n=n, dt=0.01, R=R, n_scales=N, precision="f32s"))
+    poly, scr = sobol_inputs(r, 80 + r)
+    f.init_nodes(poly, scr, np.zeros(r))
+    u, _ = f.get_nodes()
+    p = oracle_problem("cubic", r, n, 0.01, R, N)
+    rng = np.random.default_rng(r + n)
+    lw = (-spread * rng.random(n)).astype(np.float32)
+    lw[rng.random(n) < 0.1] = -np.inf
+    lw[n // 2] = 0.0
+    centre = rng.standard_normal(r)
+    f.set_state(centre, lw, 0.0, 1)
+    before = f.launches()
+    f.predict()
+    assert f.launches() - before >= 3
+    pred, off = f.get_log_weights()
+    prep = F.prepare(p, u, centre)
+    lw64 = lw.astype(np.float64)
+    Lj = F.kernel_lse(p, prep, lw64)
+    ref, _ = F.combine(p, Lj, lw64, prep.mask)
+    got = pred.astype(np.float64) + off
+    both = np.isfinite(got) == np.isfinite(ref)
+    assert both.mean() >= 0.99, np.nonzero(~both)[0][:5]
+    ok, _ = combination_err_ok(got[both], ref[both], Lj[both], p.coef, lw64[both], 1e-5)
+    assert ok
