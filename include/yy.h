@@ -83,16 +83,16 @@ typedef enum { YY_MODEL_CUBIC = 0, YY_MODEL_LINEAR = 1, YY_MODEL_PAPER_E1 = 2 } 
 typedef enum { YY_NODES_SOBOL = 0, YY_NODES_HALTON = 1, YY_NODES_FAURE = 2 } yy_nodes;
 
 /* Arithmetic of the prediction step.  FP64: every step in float64.  FP32: exact
- * float32 differences over every pair (at r >= 128 a pair whose term is provably zero in
- * float32 next to the largest of its row is not summed to the end).  BF16: a tcgen05 BF16 Gram product screens out pairs
- * whose kernel term is provably negligible, and the remaining pairs are evaluated exactly
- * in float32 (results agree with FP32 within float32 rounding).  FP32_SCREEN: the same kind
- * of screen on the FMA pipes, no tensor cores: a tile of pairs is skipped when a lower bound of
- * every live pair's squared distance over the first 64 k coordinates (k = screen_prefix,
- * default half of the 64-coordinate chunks; no screen where it cannot pay: r < 64, or r < 128
- * with n < 4096) exceeds the row's screening
- * radius; every other tile is evaluated exactly as in FP32 (results agree with FP32 within
- * float32 rounding).  Not accepted by batches. */
+ * float32 differences over every pair (at r >= 128, with n <= 512 at r >= 512, a pair whose
+ * term is provably zero in float32 next to the largest of its row is not summed to the end).
+ * BF16: a tcgen05 BF16 Gram product screens out pairs whose kernel term is provably
+ * negligible, and the remaining pairs are evaluated exactly in float32 (results agree with
+ * FP32 within float32 rounding).  FP32_SCREEN: the same kind of screen on the FMA pipes, no
+ * tensor cores: a tile of pairs is skipped when a lower bound of every live pair's squared
+ * distance over the first 64 k coordinates (k = screen_prefix, default half of the
+ * 64-coordinate chunks; no screen where it cannot pay: r < 64, or r < 128 with n < 4096)
+ * exceeds the row's screening radius; every other tile is evaluated exactly as in FP32
+ * (results agree with FP32 within float32 rounding).  Not accepted by batches. */
 typedef enum { YY_PREC_FP64 = 0, YY_PREC_FP32 = 1, YY_PREC_BF16 = 2, YY_PREC_FP32_SCREEN = 3 } yy_precision;
 
 /* Log-weights after a restart ("Local Resampling-Restart Mechanism" only says that the

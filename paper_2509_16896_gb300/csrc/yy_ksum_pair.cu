@@ -129,7 +129,12 @@ __global__ void __launch_bounds__(THREADS, BLOCKS_PER_SM) kb_pair(const Traj<flo
 // weights of a restart 175 us (tiles given up after 192 to 256 coordinates; 300 us while the
 // rows' own pairs kept their tiles), weights of an update 95 us (one heavy node; 350 us before
 // thin tiles).
-constexpr int kSkipMinDim = 128;
+// With at most 512 sources a prediction waits out one stage after the other, and the reference
+// pass and the tests add a quarter to it: measured at n <= 512, us, full form -> skipping, weights of a
+// restart / nothing to skip: r = 128 29 -> 42 / 42, r = 200 35 -> 41 / 50, r = 300 43 -> 43 / 63, r =
+// 500 59 -> 50 / 89, r = 1000 98 -> 51 / 150; so rows of 512 and more skip there.
+constexpr int kSkipMinDim = 128, kSkipMinDimSmall = 512;
+constexpr long long kSkipSmall = 512;
 constexpr size_t kMaxMaskBytes = 32768;   // ranges of up to a million sources
 constexpr float kSkipGap = 110.0f;
 
@@ -180,7 +185,7 @@ cudaError_t launch_skip_n(const Consts<float>& k, const Bufs<float>& b, int S, f
 }
 template <int N, bool NOISE>
 cudaError_t launch_n(const Consts<float>& k, const Bufs<float>& b, int S, cudaStream_t s, int* l) {
-    if (!NOISE && k.r >= kSkipMinDim && pair_skip_fits(k, b)) {
+    if (!NOISE && k.r >= (k.n > kSkipSmall ? kSkipMinDim : kSkipMinDimSmall) && pair_skip_fits(k, b)) {
         if (l) *l += 1;
         const cudaError_t e = launch_ref_n<N>(k, b, s);
         return e == cudaSuccess ? launch_skip_n<N>(k, b, S, kSkipGap, nullptr, 0, s) : e;

@@ -191,3 +191,10 @@ def test_float32_screen_of_mid_rows(yy_lib, r, n, N, R, spread):
     assert both.mean() >= 0.99, np.nonzero(~both)[0][:5]
     ok, _ = combination_err_ok(got[both], ref[both], Lj[both], p.coef, lw64[both], 1e-5)
     assert ok
+
+
+@pytest.mark.parametrize("r,n,N", [(200, 512, 2), (200, 513, 2), (511, 512, 1), (512, 512, 3), (700, 100, 2)])
+@pytest.mark.parametrize("spread", [0.0, 3000.0])
+def test_long_rows_with_few_sources(yy_lib, r, n, N, spread):
+    """Both sides of the rule that leaves the skipping form out where there are few sources."""
+    test_long_rows_with_spread_weights(yy_lib, "f32", r, n, N, spread)
