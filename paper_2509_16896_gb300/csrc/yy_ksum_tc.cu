@@ -524,9 +524,11 @@ __device__ __forceinline__ float* part_slot(const Bufs<float>& b, long long i, i
 // CTAs' marks.  Everything else -- screening, exact evaluation, row states -- is per CTA
 // and identical to the single-CTA kernel.
 // BATCH: the work list spans the filters of a batch (descriptors and TMA maps in global memory).
-// Only this instance takes the short rows' exact pairs through pair_sums_call: a call costs the
-// screening loop registers (with it the single filters' instances spilled: r = 100 prediction 90
-// -> 109 us, r = 1000 0.68 -> 0.81 ms), and it is batches that have many of them.
+// This instance takes the short rows' exact pairs through pair_sums_staged, which fits the
+// registers the screening loop leaves (no spills; a function call there, or loads a stage ahead,
+// spilled 200 to 300 bytes and cost batches of long rows up to a fifth: 8 members of r = 100, n =
+// 8192 181 -> 217 us).  Eight members, word by word -> so: r = 64, n = 8192 0.88 -> 0.44 ms, r = 50 3.91
+// -> 1.46 ms, r = 20, n = 4096 17.2 -> 7.7 ms.
 template <int N, int BN, bool PAIR, bool BATCH>
 // One CTA per SM; with 10 warps two of the four SM sub-partitions hold three warps each, so
 // the register budget is 168 per thread.
@@ -1071,10 +1073,8 @@ __global__ void __launch_bounds__(tc::NUM_THREADS, 1)
                             const long long src = sb + c;
                             const float* us = b.u + (size_t)src * k.r_pad;
                             float s1 = 0.f, s2 = 0.f;
-                            if (BATCH && b.store_f) {   // (loads a stage ahead instead of a word at a time)
-                                const float2 s12 = pair_sums_call(ut, b.f + (size_t)i * k.r_pad, us, k.r_pad);
-                                s1 = s12.x;
-                                s2 = s12.y;
+                            if (BATCH && b.store_f) {   // (16 coordinates' loads at a time)
+                                pair_sums_staged(ut, b.f + (size_t)i * k.r_pad, us, k.r, s1, s2);
                             } else {
                                 for (int d = 0; d < k.r; ++d) {
                                     const float dl = ut[d] - us[d];
