@@ -35,17 +35,18 @@ __global__ void __launch_bounds__(THREADS, BLOCKS_PER_SM)
 // bit per tile of 128 sources (fwords words per block), or nullptr.
 template <int N>
 __global__ void __launch_bounds__(THREADS, BLOCKS_PER_SM)
-    k_pair_skip(const __grid_constant__ Consts<float> k, const __grid_constant__ Bufs<float> b, int nsplit, float gap,
-                const uint32_t* __restrict__ flags, int fwords) {
+    k_pair_skip(const __grid_constant__ Consts<float> k, const __grid_constant__ Bufs<float> b, int nsplit,
+                const __grid_constant__ SkipTest skip, const uint32_t* __restrict__ flags, int fwords) {
     extern __shared__ __align__(16) float pair_smem[];
     const long long i0 = k.row0 + (long long)(blockIdx.x / nsplit) * BM;
-    block<N, false, false, true>(k, b, i0, (int)(blockIdx.x % nsplit), nsplit, pair_smem, gap,
+    block<N, false, false, true>(k, b, i0, (int)(blockIdx.x % nsplit), nsplit, pair_smem, &skip,
                                  flags ? flags + (size_t)(i0 / BM) * fwords : nullptr);
 }
 
 // Lower bounds of every target row's largest score, per scale: the larger of the row's own
 // term (u_i - u_i = 0) and its exact score against the live source of the largest log-weight.
-// Each block finds that source for itself (n words from L2); then one warp per row.
+// The second is taken down by what its rounding and the pair loop's, which adds up in
+// another order, can differ by (see yy_pair.cuh).  Each block finds that source for itself (n words from L2); then one warp per row.
 template <int N>
 __global__ void __launch_bounds__(256) k_pair_ref(const __grid_constant__ Consts<float> k,
                                                   const __grid_constant__ Bufs<float> b) {
@@ -84,11 +85,12 @@ __global__ void __launch_bounds__(256) k_pair_ref(const __grid_constant__ Consts
             s2 += __shfl_xor_sync(0xffffffffu, s2, o);
         }
         if (lane == 0) {
-            const float nf = b.nf[i], li = b.logw[i];
+            const float nf = b.nf[i], li = b.logw[i], gam = skip_gamma(k.r);
 #pragma unroll
             for (int j = 0; j < N; ++j) {
-                const float rc = -0.5f * k.tau[j] * nf;
-                b.pair_ref[(size_t)i * kMaxScales + j] = fmaxf(rc + li, fmaf(-s1, k.inv2tau[j], s2) + (rc + m));
+                const float rc = __fmul_rn(-0.5f * k.tau[j], nf);   // rounded as in the pair loop
+                const float err = gam * (5.0f * s1 * k.inv2tau[j] - 4.0f * rc) + 1e-6f * fabsf(m);
+                b.pair_ref[(size_t)i * kMaxScales + j] = fmaxf(rc + li, fmaf(-s1, k.inv2tau[j], s2) + (rc + m) - err);
             }
         }
     }
@@ -178,7 +180,9 @@ template <int N>
 cudaError_t launch_skip_n(const Consts<float>& k, const Bufs<float>& b, int S, float gap, const uint32_t* flags,
                           int fwords, cudaStream_t s) {
     const unsigned grid = (unsigned)((k.row1 - k.row0 + BM - 1) / BM * S);
-    k_pair_skip<N><<<grid, THREADS, smem_bytes<N, false, false, true>() + mask_bytes(k.n, S), s>>>(k, b, S, gap, flags,
+    SkipTest t{gap, skip_gamma(k.r), {}};
+    for (int j = 0; j < k.N; ++j) t.i2t[j] = k.inv2tau[j] * std::max(1.0f - 5.0f * t.gam, 0.0f);
+    k_pair_skip<N><<<grid, THREADS, smem_bytes<N, false, false, true>() + mask_bytes(k.n, S), s>>>(k, b, S, t, flags,
                                                                                                   fwords);
     const cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? merge_n<N, false>(k, b, S, s) : e;

@@ -112,6 +112,14 @@ __device__ __forceinline__ float max_nan(float a, float b) {
 constexpr float kZeroGap = 105.0f;
 
 constexpr int kThinGroups = 2;
+// Bound of a chain of r products' rounding, relative to the sum of their magnitudes (and of the
+// few operations around it).
+__host__ __device__ __forceinline__ float skip_gamma(int r) { return (float)(r + 16) * 6.03e-8f; }
+// What the skipping form tests with (a kernel parameter: a register per value would spill).
+struct SkipTest {
+    float gap, gam;           // nats below the reference; skip_gamma
+    float i2t[kMaxScales];    // 1 / (2 tau_j), shrunk by 5 gamma
+};
 // One block: targets i0 .. i0 + BM - 1 against the groups of 64 sources in the range [split /
 // nsplit, (split + 1) / nsplit), TN / 4 groups per source tile.  nsplit > 1: the rows' (max,
 // sum) go to b.simt_part and a merge kernel applies the combination.  OP: every pair's score
@@ -120,8 +128,12 @@ constexpr int kThinGroups = 2;
 //
 // SKIP: terms that provably cannot count are not evaluated.  b.pair_ref[i][j] is a lower bound
 // of row i's largest score at scale j (k_pair_ref); a pair whose score is below it by more than
-// gap at every scale is dropped.  Since a score is ell_s minus a sum of squares over the
-// coordinates, two bounds need no slack but rounding's (gap has 5 nats to spare):
+// gap at every scale is dropped.  A score is ell_s minus a sum of squares over the coordinates,
+// S1 / (2 tau) - S2 + Q of them with Q = tau |f_i|^2 / 2, so a part of the sum bounds it from above up
+// to rounding.  That is at most skip_gamma = (r + 16) u times the magnitudes, u = 2^-24, and |D||f| <= D^2 / (2
+// tau) + tau f^2 / 2: a computed score exceeds the bound computed on the way, the thresholds' own
+// rounding included, by less than 5 gamma S1 / (2 tau) + 8 gamma Q + 16 u |ref|.  The first is taken off by
+// shrinking 1 / (2 tau) in the test, the others from the threshold.  Two bounds are tested:
 //   - a chain's group of 4 sources is left out when its largest ell_s is below the block's lowest
 //     threshold (weights spread over many nats: the large-scale model after an update); the
 //     remaining groups of a chain keep their order;
@@ -134,7 +146,7 @@ constexpr int kThinGroups = 2;
 // flagged for this target block ([tile of 128 sources] bits) are taken.
 template <int N, bool NOISE, bool OP, bool SKIP = false>
 __device__ __forceinline__ void block(const Consts<float>& k, const Bufs<float>& b, long long i0, int split,
-                                      int nsplit, float* smem, float gap = 0.f, const uint32_t* flags = nullptr) {
+                                      int nsplit, float* smem, const SkipTest* skip = nullptr, const uint32_t* flags = nullptr) {
     static_assert(!SKIP || (!NOISE && !OP), "the skipping form is the plain one");
     constexpr int SW = stage_words<NOISE>();
     constexpr int RP = TM / 2;   // row pairs per thread
@@ -240,7 +252,11 @@ __device__ __forceinline__ void block(const Consts<float>& k, const Bufs<float>&
             const bool target = i < k.n && !b.mask[i];
 #pragma unroll
             for (int j = 0; j < N; ++j) {
-                const float v = target ? b.pair_ref[(size_t)i * kMaxScales + j] - gap : INFINITY;
+                float v = INFINITY;
+                if (target) {
+                    const float ref = b.pair_ref[(size_t)i * kMaxScales + j];
+                    v = ref - (skip->gap + 8.0f * skip->gam * (0.5f * k.tau[j] * b.nf[i]) + 1e-6f * fabsf(ref));
+                }
                 thr[tid * N + j] = v;
                 lo = (v != v) ? -INFINITY : fminf(lo, v);   // an undefined bound drops nothing
             }
@@ -419,7 +435,7 @@ __device__ __forceinline__ void block(const Consts<float>& k, const Bufs<float>&
                         float m = -INFINITY;
 #pragma unroll
                         for (int e = 0; e < TN; ++e)
-                            if (!((e & 3) == a && (e >> 2) == own)) m = max_nan(m, fmaf(-lane2(S1[a >> 1][e], a & 1), k.inv2tau[j], lane2(S2[a >> 1][e], a & 1)) + ls[e]);
+                            if (!((e & 3) == a && (e >> 2) == own)) m = max_nan(m, fmaf(-lane2(S1[a >> 1][e], a & 1), skip->i2t[j], lane2(S2[a >> 1][e], a & 1)) + ls[e]);
                         alive |= !(m < thr[(ty * 4 + a) * N + j]);
                     }
                 if (!__syncthreads_or(alive)) {

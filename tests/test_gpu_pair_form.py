@@ -198,3 +198,51 @@ def test_float32_screen_of_mid_rows(yy_lib, r, n, N, R, spread):
 def test_long_rows_with_few_sources(yy_lib, r, n, N, spread):
     """Both sides of the rule that leaves the skipping form out where there are few sources."""
     test_long_rows_with_spread_weights(yy_lib, "f32", r, n, N, spread)
+
+
+@pytest.mark.parametrize("prec", ["f32", "f32s"])
+@pytest.mark.parametrize("r,flat,n,N,dt,R", [(130, 0, 1000, 2, 1e-2, 0.3), (1000, 0, 700, 3, 1e-4, 0.3),
+                                             (1000, 500, 1281, 1, 1e-8, 0.3), (300, 150, 897, 1, 1e-9, 1.0),
+                                             (256, 100, 897, 1, 1e-9, 1.0), (256, 100, 929, 1, 1e-9, 1.0),
+                                             (256, 100, 961, 1, 1e-9, 1.0), (256, 100, 993, 1, 1e-9, 1.0), (130, 0, 16384, 2, 1e-2, 0.3),
+                                             (130, 0, 20000, 1, 1e-3, 0.3), (256, 100, 20000, 1, 1e-8, 0.5)])
+@pytest.mark.parametrize("spread", [0.0, 1.0, 30.0])
+def test_skipping_leaves_every_bit(yy_lib, prec, r, flat, n, N, dt, R, spread):
+    """Long rows leave out only terms that are zero in float32: the prediction is, bit for bit,
+    that of the form with noise coefficients, which takes every pair, at coefficients of one
+    (the metric is one, its determinant's logarithm zero; linear drift, whose preparation is the
+    same code for both).  The last `flat` coordinates have a box of no width to speak of, so that
+    the sum is all there when it is tested, and n is 32 k + 1, so that the last block of targets has
+    a row that nothing else keeps.  Steps so short that scores are 1e10 nats and their float32
+    rounding is thousands, log-weights from equal to 30 times that spread; ranges of up to 313
+    groups of sources.  Behind the float32 screen terms below e^-(ln n + 20) of the row's sum are missing:
+    2e-9 of it, so 1e-6 relative (N = 1: no combination of scales to amplify it)."""
+    from paper_2509_16896_gb300 import binding
+    if prec == "f32s" and N > 1:
+        N = 1
+    one = dict(u=1.0, u_kappa=0.0, u_zero=0, v=1.0, v_kappa=0.0)
+    poly, scr = sobol_inputs(r, 90)
+    rng = np.random.default_rng(r + n)
+    centre = rng.standard_normal(r)
+    lw = (-spread * r * R * R / (3.0 * dt) * rng.random(n)).astype(np.float32)
+    lw[rng.random(n) < 0.3] = -np.inf
+    lw[n // 2] = 0.0
+    half = np.full(r, R)
+    half[r - flat:] = R * 1e-9
+    out = []
+    for p, nz in ((prec, None), ("f32", one)):
+        f = binding.Filter(binding.make_config(model="linear", r=r, n=n, dt=dt, R=R, n_scales=N, precision=p, noise=nz))
+        f.init_nodes(poly, scr, np.zeros(r), halfwidth=half)
+        f.set_state(centre, lw, 0.0, 1)
+        f.predict()
+        lp, off = f.get_log_weights()
+        out.append((lp, off))
+    (a, oa), (b, ob) = out
+    assert oa == ob
+    assert np.isfinite(b).mean() >= 0.5 or N == 2
+    if prec == "f32":
+        assert np.array_equal(a, b)
+    else:
+        fin = np.isfinite(b)
+        assert np.array_equal(fin, np.isfinite(a))
+        assert np.all(np.abs(a[fin] - b[fin]) <= 1e-6 * np.maximum(1.0, np.abs(b[fin])))
