@@ -7,7 +7,7 @@ amplifies (`combination_err_ok`)."""
 import numpy as np
 import pytest
 
-from ._helpers import combination_err_ok, oracle_problem, sobol_inputs
+from ._helpers import combination_err_ok, oracle_problem, rel_err, sobol_inputs
 
 pytestmark = pytest.mark.gpu
 
@@ -246,3 +246,28 @@ def test_skipping_leaves_every_bit(yy_lib, prec, r, flat, n, N, dt, R, spread):
         fin = np.isfinite(b)
         assert np.array_equal(fin, np.isfinite(a))
         assert np.all(np.abs(a[fin] - b[fin]) <= 1e-6 * np.maximum(1.0, np.abs(b[fin])))
+
+
+@pytest.mark.parametrize("r,n,N,prefix", [(129, 1000, 2, 1), (191, 2049, 1, 3), (257, 1500, 3, 2), (300, 1025, 2, 5),
+                                          (1000, 1500, 3, 16)])
+@pytest.mark.parametrize("spread", [0.0, 60.0])
+def test_float32_screen_first_pass_lengths(yy_lib, r, n, N, prefix, spread):
+    """The float32 screen of long ragged rows at explicit lengths of its first pass (up to all
+    coordinates): the plain form's prediction within the terms the screen may leave out."""
+    from paper_2509_16896_gb300 import binding
+    poly, scr = sobol_inputs(r, 95)
+    rng = np.random.default_rng(r + n)
+    centre = rng.standard_normal(r)
+    lw = (-spread * rng.random(n)).astype(np.float32)
+    lw[rng.random(n) < 0.1] = -np.inf
+    lw[n // 2] = 0.0
+    out = []
+    for prec in ("f32", "f32s"):
+        f = binding.Filter(binding.make_config(model="cubic", r=r, n=n, dt=0.01, R=0.3, n_scales=N, precision=prec,
+                                               screen_prefix=prefix))
+        f.init_nodes(poly, scr, np.zeros(r))
+        f.set_state(centre, lw, 0.0, 1)
+        f.predict()
+        lp, off = f.get_log_weights()
+        out.append(lp.astype(np.float64) + off)
+    assert rel_err(out[1], out[0]) <= 2e-6

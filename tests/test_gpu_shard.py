@@ -70,6 +70,15 @@ def test_shards_match_whole_filter(yy_lib, prec, r, n, N, G):
             assert s.restart(mode=0, report=True) == did
 
 
+@pytest.mark.parametrize("prec,r,n,N,G", [("f32s", 130, 2500, 2, 2), ("f32s", 200, 4096, 3, 4), ("f32", 130, 2500, 2, 2),
+                                          ("f32", 300, 3000, 1, 4), ("f32s", 64, 5000, 1, 2)])
+def test_shards_of_long_rows_match_whole_filter(yy_lib, prec, r, n, N, G):
+    """Rows long enough for the float32 screen and for the plain form that leaves terms out: target
+    windows that start within the Gram pass's block triangle, flags and references of absolute
+    rows, a shard's own number of source ranges."""
+    test_shards_match_whole_filter(yy_lib, prec, r, n, N, G)
+
+
 def test_shard_calls_are_checked(yy_lib):
     import torch
     from paper_2509_16896_gb300 import binding
