@@ -196,7 +196,7 @@ cudaError_t prepare_ksum_f64();
 cudaError_t launch_ksum_f64(const Consts<double>& k, const Bufs<double>& b, cudaStream_t s, int* launches);
 cudaError_t launch_pair(const Consts<float>& k, const Bufs<float>& b, cudaStream_t s, int* launches);
 cudaError_t prepare_pair();
-bool pair_skip_fits(const Consts<float>& k, const Bufs<float>& b);
+bool pair_skip_fits(const Consts<float>& k, const Bufs<float>& b, bool screened);
 cudaError_t launch_pair_ref(const Consts<float>& k, const Bufs<float>& b, cudaStream_t s);
 cudaError_t launch_pair_flagged(const Consts<float>& k, const Bufs<float>& b, float gap, const uint32_t* flags,
                                 int fwords, cudaStream_t s, int* launches);

@@ -137,7 +137,11 @@ __global__ void __launch_bounds__(THREADS, BLOCKS_PER_SM) kb_pair(const Traj<flo
 // 500 59 -> 50 / 89, r = 1000 98 -> 51 / 150; so rows of 512 and more skip there.
 constexpr int kSkipMinDim = 128, kSkipMinDimSmall = 512;
 constexpr long long kSkipSmall = 512;
-constexpr size_t kMaxMaskBytes = 32768;   // ranges of up to a million sources
+// Masks of a source range: one million sources in the plain form, which has another way; behind the
+// screen as much as a block can have (ranges of 5 million), as all pairs of so many rows would take
+// minutes.
+constexpr size_t kMaxMaskBytes = 32768;
+constexpr size_t kMaxMaskBytesScreen = 160 * 1024;
 constexpr float kSkipGap = 110.0f;
 
 // Source ranges per target row (at most kSimtMaxSplit, none beyond the source groups): two
@@ -157,7 +161,7 @@ cudaError_t set_attr_n() {
     const auto a = cudaFuncAttributeMaxDynamicSharedMemorySize;
     cudaError_t e = cudaFuncSetAttribute(k_pair<N, false>, a, (int)smem_bytes<N, false, false>());
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_pair<N, true>, a, (int)smem_bytes<N, true, false>());
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_pair_skip<N>, a, (int)(smem_bytes<N, false, false, true>() + kMaxMaskBytes));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_pair_skip<N>, a, (int)(smem_bytes<N, false, false, true>() + kMaxMaskBytesScreen));
     if (e == cudaSuccess) e = cudaFuncSetAttribute(kb_pair<N>, a, (int)smem_bytes<N, false, false>());
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_op_build<N>, a, (int)smem_bytes<N, false, true>());
     return e;
@@ -189,7 +193,7 @@ cudaError_t launch_skip_n(const Consts<float>& k, const Bufs<float>& b, int S, f
 }
 template <int N, bool NOISE>
 cudaError_t launch_n(const Consts<float>& k, const Bufs<float>& b, int S, cudaStream_t s, int* l) {
-    if (!NOISE && k.r >= (k.n > kSkipSmall ? kSkipMinDim : kSkipMinDimSmall) && pair_skip_fits(k, b)) {
+    if (!NOISE && k.r >= (k.n > kSkipSmall ? kSkipMinDim : kSkipMinDimSmall) && pair_skip_fits(k, b, false)) {
         if (l) *l += 1;
         const cudaError_t e = launch_ref_n<N>(k, b, s);
         return e == cudaSuccess ? launch_skip_n<N>(k, b, S, kSkipGap, nullptr, 0, s) : e;
@@ -228,8 +232,9 @@ cudaError_t launch_pair(const Consts<float>& k, const Bufs<float>& b, cudaStream
 }
 
 // The masks of a source range fit the skipping form's shared memory.
-bool pair_skip_fits(const Consts<float>& k, const Bufs<float>& b) {
-    return b.pair_ref && mask_bytes(k.n, pair_splits(k, b, k.row1 - k.row0)) <= kMaxMaskBytes;
+bool pair_skip_fits(const Consts<float>& k, const Bufs<float>& b, bool screened) {
+    return b.pair_ref && mask_bytes(k.n, pair_splits(k, b, k.row1 - k.row0)) <=
+                             (screened ? kMaxMaskBytesScreen : kMaxMaskBytes);
 }
 
 cudaError_t launch_pair_ref(const Consts<float>& k, const Bufs<float>& b, cudaStream_t s) {

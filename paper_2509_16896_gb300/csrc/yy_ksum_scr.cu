@@ -38,7 +38,7 @@ __global__ void __launch_bounds__(THREADS, 4)
     __shared__ __align__(16) float st[2 * GSW];
     __shared__ float rho_r[GM], rho_c[GN], q_r[GM], q_c[GN], red[8];
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4, lane = tid & 31, wib = tid >> 5;
-    const int ta = blockIdx.y, tc = blockIdx.x;   // block of 64 rows, tile of 128 columns
+    const int ta = blockIdx.x, tc = blockIdx.y;   // block of 64 rows, tile of 128 columns (up to 65535)
     if (tc < ta / 2) return;                      // its pairs belong to the block with the roles swapped
     const long long i0 = (long long)ta * GM, c0 = (long long)tc * GN;
     const bool rows_in = i0 < k.row1 && i0 + GM > k.row0, cols_in = c0 < k.row1 && c0 + GN > k.row0;
@@ -198,7 +198,7 @@ size_t scr_flag_words(long long n_pad) { return (size_t)(n_pad / 32) * (size_t)(
 // First pass over at most k1 coordinates (a multiple of 64: the norms come in chunks of 64),
 // then exact evaluation of every flagged tile.
 cudaError_t launch_ksum_scr32(const Consts<float>& k, const Bufs<float>& b, int k1, cudaStream_t s, int* launches) {
-    if (!screen_pays(k) || !pair_skip_fits(k, b)) return launch_pair(k, b, s, launches);
+    if (!screen_pays(k) || !pair_skip_fits(k, b, true)) return launch_pair(k, b, s, launches);
     if (!b.nu_chunk || !b.scr_flags) return cudaErrorInvalidValue;
     k1 = std::max(64, std::min((k1 + 63) / 64 * 64, k.r_pad));
     const float T = logf((float)k.n) + 20.0f;
@@ -206,7 +206,7 @@ cudaError_t launch_ksum_scr32(const Consts<float>& k, const Bufs<float>& b, int 
     cudaError_t e = cudaMemsetAsync(b.scr_flags, 0, scr_flag_words(k.n_pad) * sizeof(uint32_t), s);
     if (e != cudaSuccess) return e;
     if ((e = launch_pair_ref(k, b, s)) != cudaSuccess) return e;
-    const dim3 grid((unsigned)(k.n_pad / GN), (unsigned)(k.n_pad / GM));
+    const dim3 grid((unsigned)(k.n_pad / GM), (unsigned)(k.n_pad / GN));
     switch (k.N) {
         case 1: k_scr_gram<1><<<grid, THREADS, 0, s>>>(k, b, k1, T, b.scr_flags, fwords); break;
         case 2: k_scr_gram<2><<<grid, THREADS, 0, s>>>(k, b, k1, T, b.scr_flags, fwords); break;
