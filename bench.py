@@ -191,6 +191,35 @@ def _gram_flops(r, k, stage, tiles, resc, bn=256):
     return 2.0 * 128 * bn * (tiles * min(stage * k, r_pad) + resc * r_pad)
 
 
+def _takes_every_pair(r, n, prec):
+    """Whether the prediction on the CUDA cores evaluates all n^2 pairs over all coordinates.
+    Longer rows of the float32 forms leave out terms that cannot count (include/yy.h,
+    yy_precision), short rows of the float64 form select theirs in float32."""
+    if prec == "f32":
+        return r < (128 if n > 512 else 512)
+    if prec == "f32s":
+        return r < 64 or (r < 128 and n < 4096)
+    return prec == "f64" and r > 64
+
+
+def _alu_roofline(r, n, prec, pred_ms):
+    """Roofline of a prediction on the CUDA cores: 3 n^2 r operations against the FP32 pipe where
+    every pair is evaluated in float32.  Elsewhere the operations done are not counted, so there is
+    no rate and no fraction, only what a prediction covers."""
+    flops = 3.0 * n * n * r
+    full = prec != "f64" and _takes_every_pair(r, n, prec)
+    kernel = {"f32": "k_pair" if full else "k_pair_skip", "f32s": "k_pair" if full else "k_scr_gram + k_pair_skip",
+              "f64": "k_ksum_simt<double>" if r > 64 else "k_ksum_f64"}[prec]
+    roof = {"bound": "alu", "achieved": round(flops / (pred_ms / 1e3) / 1e12, 3) if full else None,
+            "peak": _fma_peak() if full else None, "unit": "TFLOP/s", "kernel": kernel + " (difference form)",
+            "kernel_ms": round(pred_ms, 4), ("algorithmic" if full else "covered") + "_flops_per_launch": flops}
+    if full:
+        roof["peak_source"] = "derived: 152 SMs x 128 FP32 lanes x 2 flops x max SM clock"
+    else:
+        roof["note"] = "terms that cannot count are left out; the operations done are not counted"
+    return roof
+
+
 def _config(w, prec, screen_type):
     return {"workload": w.name, "r": w.r, "n": w.n, "n_scales": w.n_scales, "dt": w.dt,
             "R": w.R, "restart_interval": w.restart_interval, "ess_frac": w.ess_frac,
@@ -284,12 +313,8 @@ def measure_single(w, prec, screen_type, screen_prefix, K, W, device, seed, dist
                 "unit": "TFLOP/s", "kernel": "k_ksum_tc (screen Gram products of the prediction)",
                 "kernel_ms": round(pred_ms, 4), "algorithmic_flops_per_launch": flops, "peak_source": note}
     else:
-        flops = 3.0 * w.n * w.n * w.r
-        roof = {"bound": "alu", "achieved": round(flops / (pred_ms / 1e3) / 1e12, 3), "peak": _fma_peak(),
-                "unit": "TFLOP/s", "kernel": "k_pair / k_pair_skip (difference form)", "kernel_ms": round(pred_ms, 4),
-                "algorithmic_flops_per_launch": flops,
-                "peak_source": "derived: 152 SMs x 128 FP32 lanes x 2 flops x max SM clock"}
-    roof["frac"] = round(roof["achieved"] / roof["peak"], 4)
+        roof = _alu_roofline(w.r, w.n, prec, pred_ms)
+    roof["frac"] = round(roof["achieved"] / roof["peak"], 4) if roof["achieved"] is not None else None
     with torch.cuda.stream(stream):
         flt.update(dys[0])   # leave the handle in a consistent state
     steps_per_s = K / (t_max / 1e3)
@@ -299,8 +324,9 @@ def measure_single(w, prec, screen_type, screen_prefix, K, W, device, seed, dist
            # screen proves most of them negligible and evaluates the rest (the self terms of
            # the live nodes and the exact pairs) in float32
            "pairs_covered_per_step": float(w.n_scales) * w.n * w.n,
+           # (the forms that leave terms out on the CUDA cores do not count them: None)
            "pairs_evaluated_per_step": float(w.n_scales) * (live + exact) if prec == "bf16" else
-                                       float(w.n_scales) * w.n * w.n}
+                                       float(w.n_scales) * w.n * w.n if _takes_every_pair(w.r, w.n, prec) else None}
     return res, flt, tr, stream
 
 
@@ -330,13 +356,13 @@ def _time_precision(w, prec, steps, warmup, tr, device, screen_prefix=0):
 
 
 def _comparators(w, K, W, tr, device, fp32_steps, est):
-    """The plain FP32 GPU form (difference form) and the screened FP32 form
-    (the same kind of screen with its bound on the FMA pipes), each with its RMSE next to
-    the mixed path's on the same steps: the first isolates pruning + precision, the second
-    precision alone."""
+    """The plain FP32 GPU form (difference form; long rows leave out the terms that are zero in
+    float32, so it is not a count of every pair's work) and the screened FP32 form (the same
+    kind of screen with its bound on the FMA pipes), each with its RMSE next to the mixed
+    path's on the same steps."""
     S = min(fp32_steps, K)
     out = {}
-    for key, prec in (("fp32_dense", "f32"), ("fp32_screened", "f32s")):
+    for key, prec in (("fp32_plain", "f32"), ("fp32_screened", "f32s")):
         c = _time_precision(w, prec, S, W, tr, device)
         c["rmse_mixed_same_steps"] = _rmse(est[:S], tr.x[W:W + S])
         out[key] = c
@@ -466,7 +492,8 @@ def run_yy(args):
         "data": "synthetic (seeded Euler-Maruyama cubic sensor, scrambled Sobol nodes)",
         "config": _config(w, prec, args.screen_type),
         "pairs_covered_per_s": round(steps_per_s * res["pairs_covered_per_step"], 1),
-        "pairs_evaluated_per_s": round(steps_per_s * res["pairs_evaluated_per_step"], 1),
+        "pairs_evaluated_per_s": round(steps_per_s * res["pairs_evaluated_per_step"], 1)
+                                 if res["pairs_evaluated_per_step"] is not None else None,
         "rmse": res["rmse"],
         "restarts": res["restarts"],
         "clocks": res["clocks"],
