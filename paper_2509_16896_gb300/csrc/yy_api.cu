@@ -203,7 +203,7 @@ size_t carve(const yy_config* c, char* base, Bufs<T>* out) {
     // ranges' partial states
     if (c->precision != YY_PREC_BF16 && n_pad < 2 * kSms * 64)
         b.simt_part = cv.take<T>((size_t)n_pad * kSimtMaxSplit * kMaxScales * 2 * sizeof(T));
-    if (c->precision == YY_PREC_FP32_SCREEN) b.scr_flags = cv.take<uint32_t>(scr_flag_words(n_pad) * sizeof(uint32_t));
+    if (c->precision == YY_PREC_FP32_SCREEN) b.scr_flags = cv.take<uint32_t>(scr_flag_words(c->r, c->n, n_pad) * sizeof(uint32_t));
     if (c->precision != YY_PREC_FP64)
         b.pair_ref = cv.take<float>((size_t)n_pad * kMaxScales * sizeof(float));
     if (c->precision == YY_PREC_BF16) {

@@ -196,11 +196,11 @@ cudaError_t prepare_ksum_f64();
 cudaError_t launch_ksum_f64(const Consts<double>& k, const Bufs<double>& b, cudaStream_t s, int* launches);
 cudaError_t launch_pair(const Consts<float>& k, const Bufs<float>& b, cudaStream_t s, int* launches);
 cudaError_t prepare_pair();
-bool pair_skip_fits(const Consts<float>& k, const Bufs<float>& b, bool screened);
+bool pair_skip_fits(const Consts<float>& k, const Bufs<float>& b);
 cudaError_t launch_pair_ref(const Consts<float>& k, const Bufs<float>& b, cudaStream_t s);
 cudaError_t launch_pair_flagged(const Consts<float>& k, const Bufs<float>& b, float gap, const uint32_t* flags,
                                 int fwords, cudaStream_t s, int* launches);
-size_t scr_flag_words(long long n_pad);
+size_t scr_flag_words(int r, long long n, long long n_pad);
 cudaError_t launch_ksum_scr32(const Consts<float>& k, const Bufs<float>& b, int k1, cudaStream_t s, int* launches);
 cudaError_t launch_op_build(const Consts<float>& k, const Bufs<float>& b, bool force, cudaStream_t s);
 cudaError_t launch_op_apply(const Consts<float>& k, const Bufs<float>& b, cudaStream_t s);

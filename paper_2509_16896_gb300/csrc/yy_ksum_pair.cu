@@ -127,8 +127,8 @@ __global__ void __launch_bounds__(THREADS, BLOCKS_PER_SM) kb_pair(const Traj<flo
 
 // The skipping form: from this many coordinates (its reference pass and masks cost about 10 us,
 // and a tile is not given up before 64 coordinates: at r = 100 nothing is), up to this much
-// mask.  Measured, large-scale model at r = 1000, n = 2000, N = 2, full form 620 us per prediction:
-// weights of a restart 175 us (tiles given up after 192 to 256 coordinates; 300 us while the
+// mask.  Measured, large-scale model at r = 1000, n = 2000, N = 2, full form 545 us per prediction:
+// weights of a restart 165 us (tiles given up after 192 to 256 coordinates; 300 us while the
 // rows' own pairs kept their tiles), weights of an update 95 us (one heavy node; 350 us before
 // thin tiles).
 // With at most 512 sources a prediction waits out one stage after the other, and the reference
@@ -137,11 +137,9 @@ __global__ void __launch_bounds__(THREADS, BLOCKS_PER_SM) kb_pair(const Traj<flo
 // 500 59 -> 50 / 89, r = 1000 98 -> 51 / 150; so rows of 512 and more skip there.
 constexpr int kSkipMinDim = 128, kSkipMinDimSmall = 512;
 constexpr long long kSkipSmall = 512;
-// Masks of a source range: one million sources in the plain form, which has another way; behind the
-// screen as much as a block can have (ranges of 5 million), as all pairs of so many rows would take
-// minutes.
+// Masks of a source range: one million sources in the plain form, which has another way (behind the
+// screen kMaxMaskBytesScreen, 5 million, as all pairs of so many rows would take minutes).
 constexpr size_t kMaxMaskBytes = 32768;
-constexpr size_t kMaxMaskBytesScreen = 160 * 1024;
 constexpr float kSkipGap = 110.0f;
 
 // Source ranges per target row (at most kSimtMaxSplit, none beyond the source groups): two
@@ -173,7 +171,6 @@ cudaError_t launch_ref_n(const Consts<float>& k, const Bufs<float>& b, cudaStrea
     k_pair_ref<N><<<(unsigned)std::min<long long>((rows + 7) / 8, 2 * kSms), 256, 0, s>>>(k, b);
     return cudaGetLastError();
 }
-size_t mask_bytes(long long n, int S) { return 16 * sizeof(uint32_t) * (size_t)mask_words(n, S); }
 
 template <int N, bool NOISE>
 cudaError_t merge_n(const Consts<float>& k, const Bufs<float>& b, int S, cudaStream_t s) {
@@ -186,14 +183,14 @@ cudaError_t launch_skip_n(const Consts<float>& k, const Bufs<float>& b, int S, f
     const unsigned grid = (unsigned)((k.row1 - k.row0 + BM - 1) / BM * S);
     SkipTest t{gap, skip_gamma(k.r), {}};
     for (int j = 0; j < k.N; ++j) t.i2t[j] = k.inv2tau[j] * std::max(1.0f - 5.0f * t.gam, 0.0f);
-    k_pair_skip<N><<<grid, THREADS, smem_bytes<N, false, false, true>() + mask_bytes(k.n, S), s>>>(k, b, S, t, flags,
+    k_pair_skip<N><<<grid, THREADS, smem_bytes<N, false, false, true>() + pair_mask_bytes(k.n, S), s>>>(k, b, S, t, flags,
                                                                                                   fwords);
     const cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? merge_n<N, false>(k, b, S, s) : e;
 }
 template <int N, bool NOISE>
 cudaError_t launch_n(const Consts<float>& k, const Bufs<float>& b, int S, cudaStream_t s, int* l) {
-    if (!NOISE && k.r >= (k.n > kSkipSmall ? kSkipMinDim : kSkipMinDimSmall) && pair_skip_fits(k, b, false)) {
+    if (!NOISE && k.r >= (k.n > kSkipSmall ? kSkipMinDim : kSkipMinDimSmall) && pair_skip_fits(k, b)) {
         if (l) *l += 1;
         const cudaError_t e = launch_ref_n<N>(k, b, s);
         return e == cudaSuccess ? launch_skip_n<N>(k, b, S, kSkipGap, nullptr, 0, s) : e;
@@ -232,9 +229,8 @@ cudaError_t launch_pair(const Consts<float>& k, const Bufs<float>& b, cudaStream
 }
 
 // The masks of a source range fit the skipping form's shared memory.
-bool pair_skip_fits(const Consts<float>& k, const Bufs<float>& b, bool screened) {
-    return b.pair_ref && mask_bytes(k.n, pair_splits(k, b, k.row1 - k.row0)) <=
-                             (screened ? kMaxMaskBytesScreen : kMaxMaskBytes);
+bool pair_skip_fits(const Consts<float>& k, const Bufs<float>& b) {
+    return b.pair_ref && pair_mask_bytes(k.n, pair_splits(k, b, k.row1 - k.row0)) <= kMaxMaskBytes;
 }
 
 cudaError_t launch_pair_ref(const Consts<float>& k, const Bufs<float>& b, cudaStream_t s) {

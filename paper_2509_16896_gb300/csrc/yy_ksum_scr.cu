@@ -191,19 +191,25 @@ __global__ void __launch_bounds__(THREADS, 4)
 // r = 64 n = 2048 60 -> 58 / 68, n = 4096 193 -> 82 / 107; r = 100 n = 2048 79 -> 67 / 118, n = 4096 277 -> 93 /
 // 304, n = 16384 3280 -> 511 / 4088; r = 127 n = 4096 331 -> 81 / 329, n = 16384 3989 -> 496 / 3826.
 // Longer rows are screened at any size: their tiles are also given up on the way.
-static bool screen_pays(const Consts<float>& k) { return k.r >= 128 || (k.r >= 64 && k.n >= 4096); }
+static bool screen_pays(int r, long long n) { return r >= 128 || (r >= 64 && n >= 4096); }
 
-size_t scr_flag_words(long long n_pad) { return (size_t)(n_pad / 32) * (size_t)((n_pad / 128 + 31) / 32); }
+// Flags of a filter that is screened: one bit per block of 32 targets and tile of 128 sources.  None (0)
+// where the plain form is what runs: see above, or beyond what the masks of one source range hold.
+size_t scr_flag_words(int r, long long n, long long n_pad) {
+    if (!screen_pays(r, n) || pair_mask_bytes(n, 1) > kMaxMaskBytesScreen) return 0;
+    return (size_t)(n_pad / 32) * (size_t)((n_pad / 128 + 31) / 32);
+}
 
 // First pass over at most k1 coordinates (a multiple of 64: the norms come in chunks of 64),
 // then exact evaluation of every flagged tile.
 cudaError_t launch_ksum_scr32(const Consts<float>& k, const Bufs<float>& b, int k1, cudaStream_t s, int* launches) {
-    if (!screen_pays(k) || !pair_skip_fits(k, b, true)) return launch_pair(k, b, s, launches);
-    if (!b.nu_chunk || !b.scr_flags) return cudaErrorInvalidValue;
+    const size_t words = scr_flag_words(k.r, k.n, k.n_pad);
+    if (words == 0) return launch_pair(k, b, s, launches);
+    if (!b.nu_chunk || !b.scr_flags || !b.pair_ref) return cudaErrorInvalidValue;
     k1 = std::max(64, std::min((k1 + 63) / 64 * 64, k.r_pad));
     const float T = logf((float)k.n) + 20.0f;
     const int fwords = (int)((k.n_pad / 128 + 31) / 32);
-    cudaError_t e = cudaMemsetAsync(b.scr_flags, 0, scr_flag_words(k.n_pad) * sizeof(uint32_t), s);
+    cudaError_t e = cudaMemsetAsync(b.scr_flags, 0, words * sizeof(uint32_t), s);
     if (e != cudaSuccess) return e;
     if ((e = launch_pair_ref(k, b, s)) != cudaSuccess) return e;
     const dim3 grid((unsigned)(k.n_pad / GM), (unsigned)(k.n_pad / GN));

@@ -17,7 +17,7 @@
 // 16384, N = 2 (6.8 ms unpacked, one word per load, 4 x 4 pairs): 8 x 8 pairs and two blocks per SM
 // 3.9 ms, 4 x 8 at three blocks 3.4 ms (FMA pipe 68 % busy, waiting on fixed latencies), at
 // four 3.3 ms = 24.4 T pair-coordinate operations a second, 0.61 of the pipe; r = 17, n = 9001,
-// N = 1: 0.62 -> 0.29 ms; r = 1000, n = 2000: 0.93 -> 0.62 ms (8 source ranges: blocks of unequal
+// N = 1: 0.62 -> 0.29 ms; r = 1000, n = 2000: 0.95 -> 0.55 ms (8 source ranges: blocks of unequal
 // number per SM).  16 coordinates per stage, double-buffered and filled by 4-byte
 // asynchronous copies that transpose on the way (coordinate-major rows padded by 4 words:
 // two-way conflicts at most); the copies of the next stage, across source tiles, run under
@@ -53,6 +53,8 @@ __host__ __device__ __forceinline__ int mask_words(long long n, int nsplit) {
     const long long groups = (n + 63) / 64;
     return (int)(((groups + nsplit - 1) / nsplit + 31) / 32);
 }
+constexpr size_t kMaxMaskBytesScreen = 160 * 1024;   // as much as a block can have
+inline size_t pair_mask_bytes(long long n, int nsplit) { return 16 * sizeof(uint32_t) * (size_t)mask_words(n, nsplit); }
 // Two stages | log-sum-exp states per thread [TM][N][2][THREADS] | source terms of two tiles |
 // |f|^2 of the targets | skipping form: thresholds [BM][N], group tables of two tiles [2][2][16],
 // four words, chain masks [16][mask_words].

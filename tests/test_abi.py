@@ -78,3 +78,14 @@ def test_workspace_grows_with_problem(lib):
     big = lib.yy_workspace_bytes(ctypes.byref(_cfg(n=65536, r=1000, precision="bf16", n_scales=3)))
     # u, f (float32) and the bf16 copy: >= 10 bytes per padded coordinate
     assert big >= 65536 * 1024 * 10 > small
+
+
+def test_screen_flags_only_where_the_screen_runs(lib):
+    """The float32 screen keeps n^2 / 32768 bytes of tile flags; a filter too short or too large for
+    the screen takes the plain form and has no use for them (12 GB at 20 million nodes)."""
+    def need(r, n, prec):
+        return lib.yy_workspace_bytes(ctypes.byref(_cfg(n=n, r=r, precision=prec)))
+    for r, n in ((10, 1_000_000), (200, 20_000_000)):
+        norms = (n + 255) // 256 * 256 * ((r + 63) // 64) * 4
+        assert need(r, n, "f32s") <= need(r, n, "f32") + norms + 4096
+    assert need(200, 1_000_000, "f32s") > need(200, 1_000_000, "f32") + 1_000_000 ** 2 // 32768
